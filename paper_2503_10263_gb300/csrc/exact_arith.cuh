@@ -1,0 +1,219 @@
+// exact_arith.cuh - correctly rounded FP64 quotients, roots and sums with few
+// instructions on the FP64 pipe.
+//
+// GB300 issues a warp's FP64 instruction over 64 cycles of its scheduler's
+// share of the pipe, an FP32 or integer one over one or two, and the kernels
+// that use these functions keep the FP64 pipe busy while most issue slots are
+// free.  Each function gives the bits of the IEEE operation it stands for:
+// an FP32 seed, two exact FP64 residuals (one fused multiply-add each) whose
+// corrections are formed in FP32 and added to the result's bits as integers,
+// and a test of the last correction's distance from a rounding boundary (the
+// residual form of P. W. Markstein, "Computation of elementary functions on
+// the IBM RISC System/6000 processor", IBM J. Res. Dev. 34, 1990).  Where the
+// test cannot decide, or an operand is outside the range treated here (zero,
+// subnormal, negative, infinite, NaN, a quotient outside the normal range),
+// the IEEE operation itself is called.
+//
+// The same source compiles for the host (the seeds are then 1/x and
+// 1/sqrt(x)), where the tests compare it with the IEEE operations; the result
+// does not depend on the seed's last bits.
+#pragma once
+#include <cmath>
+#include <cstdint>
+#include <cstring>
+
+#ifdef __CUDACC__
+#define XA_FN __device__ __forceinline__
+#else
+#define XA_FN static inline
+#ifndef XA_SEED
+#define XA_SEED(y) (y)        // tests perturb the seeds within their bound
+#endif
+#endif
+
+namespace karl {
+
+#ifdef __CUDACC__
+XA_FN long long xa_bits(double x) { return __double_as_longlong(x); }
+XA_FN double xa_dbl(long long b) { return __longlong_as_double(b); }
+XA_FN int xa_fbits(float x) { return __float_as_int(x); }
+XA_FN float xa_flt(int b) { return __int_as_float(b); }
+XA_FN double xa_fma(double a, double b, double c) { return __fma_rn(a, b, c); }
+XA_FN float xa_fmul(float a, float b) { return __fmul_rn(a, b); }
+XA_FN float xa_rcp(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+XA_FN float xa_rsqrt(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+XA_FN int xa_rint(float x) { return __float2int_rn(x); }
+XA_FN float xa_float(int n) { return __int2float_rn(n); }
+XA_FN double xa_ieee_div(double a, double b) { return __ddiv_rn(a, b); }
+XA_FN double xa_ieee_sqrt(double a) { return __dsqrt_rn(a); }
+#else
+XA_FN long long xa_bits(double x) { long long b; std::memcpy(&b, &x, 8); return b; }
+XA_FN double xa_dbl(long long b) { double x; std::memcpy(&x, &b, 8); return x; }
+XA_FN int xa_fbits(float x) { int b; std::memcpy(&b, &x, 4); return b; }
+XA_FN float xa_flt(int b) { float x; std::memcpy(&x, &b, 4); return x; }
+XA_FN double xa_fma(double a, double b, double c) { return std::fma(a, b, c); }
+XA_FN float xa_fmul(float a, float b) { return a * b; }
+XA_FN float xa_rcp(float x) { return XA_SEED(1.0f / x); }
+XA_FN float xa_rsqrt(float x) { return XA_SEED((float)(1.0 / std::sqrt((double)x))); }
+XA_FN int xa_rint(float x) { return (int)std::nearbyint(x); }
+XA_FN float xa_float(int n) { return (float)n; }
+XA_FN double xa_ieee_div(double a, double b) { return a / b; }
+XA_FN double xa_ieee_sqrt(double a) { return std::sqrt(a); }
+#endif
+
+constexpr long long XA_ONE = 0x3ff0000000000000LL;
+constexpr long long XA_MANT = 0x000fffffffffffffLL;
+
+// The significand of a double as an FP32 number in [1, 2), truncated.
+XA_FN float xa_top24(long long b) {
+  return xa_flt(0x3f800000 | ((int)(b >> 29) & 0x7fffff));
+}
+// x truncated to FP32 on the bits; |x| < 2^127, and 0 below 2^-126.
+XA_FN float xa_trunc_f(double x) {
+  const long long b = xa_bits(x);
+  const int h = (int)(b >> 32);
+  const int t = (h & 0x7fffffff) - (896 << 20);              // exponent rebiased
+  const int m = t < 0 ? 0 : (t << 3) | (int)((unsigned)b >> 29);
+  return xa_flt(m | (h & (int)0x80000000));
+}
+// An FP32 number in [2^-126, 2^127) as a double.
+XA_FN double xa_from_f(float f) {
+  return xa_dbl(((long long)xa_fbits(f) << 29) + (896LL << 52));
+}
+
+// The last correction (in units of the result's last place) lies within 0.5 of
+// the integer it is rounded to; beyond XA_TIE its FP32 error (at most 2^-11 of
+// a unit, bounded in xa_div and xa_sqrt) could change which integer is
+// nearest.  One operand pair in a thousand goes to the IEEE operation.
+constexpr float XA_TIE = 0.4995f;
+
+// a / b for b > 0, correctly rounded.  With significands m_a, m_b in [1, 2):
+// the seed r ~ 1/m_b is within 2^-22 (truncated operand 2^-23, rcp.approx
+// 1 ulp), the quotient q0 = m_a r within 2^-21.7 (the truncations of a and b
+// act against each other); the first residual's FP32 correction (relative
+// error 2^-21.2) leaves q1 within 2^-42.9, below 2^10.1 units of the last
+// place, and the second correction's error is below 2^-11 units.  q0's
+// significand must keep eight FP32 units from its binade's ends, so the
+// corrections (four of them at most) stay within it.  Two FP64 instructions.
+XA_FN double xa_div(double a, double b) {
+  const long long sa = xa_bits(a) & (long long)0x8000000000000000ULL;
+  const long long ba = xa_bits(a) ^ sa, bb = xa_bits(b);
+  const int ea = (int)(ba >> 52), eb = (int)(bb >> 52);      // eb negative with the sign bit
+  // magnitudes in (2^-500, 2^500): normal, and so is the quotient
+  if ((unsigned)(ea - 523) < 1000u && (unsigned)(eb - 523) < 1000u) {
+    const double ma = xa_dbl((ba & XA_MANT) | XA_ONE), mb = xa_dbl((bb & XA_MANT) | XA_ONE);
+    const float r = xa_rcp(xa_top24(bb));
+    const float q0f = xa_fmul(xa_top24(ba), r);              // in (0.5, 2)
+    const int qm = xa_fbits(q0f) & 0x7fffff;
+    // 2^52 or 2^53: units of the last place in q0's binade
+    const float unit = xa_fbits(q0f) < 0x3f800000 ? 9007199254740992.0f : 4503599627370496.0f;
+    const float ru = xa_fmul(r, unit);
+    const double q0 = xa_from_f(q0f);
+    const double r0 = xa_fma(-q0, mb, ma);
+    const int n0 = xa_rint(xa_fmul(xa_trunc_f(r0), xa_fmul(ru, 0.0625f)));   // units of 16
+    const long long b1 = xa_bits(q0) + ((long long)n0 << 4);
+    const double r1 = xa_fma(-xa_dbl(b1), mb, ma);
+    const float c1 = xa_fmul(xa_trunc_f(r1), ru);
+    const int n1 = xa_rint(c1);
+    const float off = c1 - xa_float(n1);
+    if ((unsigned)(qm - 8) < 0x7fffffu - 16u && off < XA_TIE && off > -XA_TIE)
+      return xa_dbl((b1 + n1 + ((long long)(ea - eb) << 52)) | sa);
+  }
+  return xa_ieee_div(a, b);
+}
+
+// sqrt(a), correctly rounded; the same scheme with m in [1, 4), a = m 4^k,
+// the seed y ~ 1/sqrt(m) (rsqrt.approx, 2^-22.3 with the truncated operand)
+// and corrections residual x y/2 (the root's second-order term is in the
+// first one's relative error, 2^-20.9; the second one's is below 2^-11 units).
+// Two FP64 instructions.
+XA_FN double xa_sqrt(double a) {
+  const long long ba = xa_bits(a);
+  const int e = (int)(ba >> 52);
+  if ((unsigned)(e - 523) < 1000u) {
+    const int odd = (e & 1) ^ 1;                             // exponent e - 1023 odd
+    const long long bm = (ba & XA_MANT) | ((long long)(1023 + odd) << 52);
+    const double m = xa_dbl(bm);
+    const float mf = xa_flt((xa_fbits(xa_top24(ba))) + (odd << 23));
+    const float y = xa_rsqrt(mf);
+    const float g0f = xa_fmul(mf, y);                        // in [1, 2)
+    const int gm = xa_fbits(g0f) & 0x7fffff;
+    const float yu = xa_fmul(y, 2251799813685248.0f);        // y/2 x 2^52
+    const double g0 = xa_from_f(g0f);
+    const double r0 = xa_fma(-g0, g0, m);
+    const int n0 = xa_rint(xa_fmul(xa_trunc_f(r0), xa_fmul(yu, 0.0625f)));
+    const long long b1 = xa_bits(g0) + ((long long)n0 << 4);
+    const double g1 = xa_dbl(b1);
+    const double r1 = xa_fma(-g1, g1, m);
+    const float c1 = xa_fmul(xa_trunc_f(r1), yu);
+    const int n1 = xa_rint(c1);
+    const float off = c1 - xa_float(n1);
+    if (g0f >= 1.0f && (unsigned)(gm - 8) < 0x7fffffu - 16u && off < XA_TIE && off > -XA_TIE)
+      return xa_dbl(b1 + n1 + ((long long)((e - odd - 1023) / 2) << 52));
+  }
+  return xa_ieee_sqrt(a);
+}
+
+// k with 1 + x = 1 + k 2^-52 rounded to nearest even, for 0 <= x < 2^-25
+// (then k < 2^27): x's significand shifted right by 1023 - e places.
+XA_FN int xa_ulps_of_1p(double x) {
+  const long long b = xa_bits(x);
+  const int s = 1023 - (int)(b >> 52);                       // 26 and up
+  if (s > 53) return 0;                                      // x 2^52 below one half
+  const long long m = (b & XA_MANT) | 0x0010000000000000LL;
+  const long long h = 1LL << (s - 1);
+  return (int)((m + h - 1 + ((m >> s) & 1)) >> s);
+}
+
+// sqrt(1 + k 2^-52), correctly rounded, is 1 + floor(k/2) 2^-52 for
+// 0 <= k < 2^27: in units of 2^-52 the root is k/2 - d with
+// 0 < d = k^2 2^-55 (1 - ...) < 1/2 (d = 0 at k = 0), so an even k rounds to
+// k/2 and an odd one, just below the midpoint, down.
+XA_FN int xa_sqrt_ulps(int k) { return k >> 1; }
+
+// a / (1 + j 2^-52), correctly rounded, for 0 <= j < 2^26 and a normal a,
+// by integers: with the significand A, the quotient is A - w,
+// w = A j / (2^52 + j) = w0 - w0 j 2^-52 + ..., w0 = A j 2^-52.  In units of
+// 2^-52, w's fraction is taken as frac(w0) - floor(w0) j, off by less than
+// 2^28; a fraction nearer to one half than that, or an A - w below 2^52,
+// goes to the IEEE division.  No FP64 instruction.
+XA_FN double xa_div_1p(double a, int j) {
+  if (j == 0) return a;
+  const long long ba = xa_bits(a);
+  const unsigned long long A = (unsigned long long)(ba & XA_MANT) | 0x0010000000000000ULL;
+  const unsigned long long p0 = (A & 0xffffffffULL) * (unsigned long long)j;
+  const unsigned long long p1 = (A >> 32) * (unsigned long long)j + (p0 >> 32);
+  const int w0 = (int)(p1 >> 20);                            // floor(A j 2^-52) < 2^27
+  const long long frac = (long long)(((p1 & 0xfffffULL) << 32) | (p0 & 0xffffffffULL));
+  const long long g = frac - (long long)w0 * j + (1LL << 51);
+  const long long n = w0 + (g >> 52);                        // w rounded to nearest
+  const long long rest = g & XA_MANT;
+  const int e = (int)(ba >> 52) & 0x7ff;
+  if (rest > (1LL << 28) && rest < (1LL << 52) - (1LL << 28) && (ba & XA_MANT) >= n &&
+      e > 0 && e < 0x7ff)
+    return xa_dbl(ba - n);
+  return xa_ieee_div(a, xa_dbl(XA_ONE + j));
+}
+
+// x / 2 and 2 x on the exponent (exact); operands near the ends of the range
+// take the multiplication.
+XA_FN double xa_half(double x) {
+  const long long b = xa_bits(x);
+  const int e = (int)(b >> 52) & 0x7ff;
+  return e > 1 && e < 0x7ff ? xa_dbl(b - (1LL << 52)) : x * 0.5;
+}
+XA_FN double xa_twice(double x) {
+  const long long b = xa_bits(x);
+  const int e = (int)(b >> 52) & 0x7ff;
+  return e > 0 && e < 0x7fe ? xa_dbl(b + (1LL << 52)) : x * 2.0;
+}
+
+}  // namespace karl

@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -193,6 +194,8 @@ struct karl_ctx {
   // full-orbit runs: primaries, the lists of two generations, raw tallies
   DevBuf<double> o_px, o_py, o_pz, o_pe, o_pmu, o_pphi, o_ez, o_energy, o_end, o_u2edge,
       o_edge2;
+  DevBuf<float2> o_bin2;
+  DevBuf<long long> o_zedge;
   DevBuf<uint8_t> o_psp, o_lsp[2];
   DevBuf<double> o_lx[2], o_ly[2], o_lz[2], o_lux[2], o_luy[2], o_luz[2];
   DevBuf<unsigned long long> o_lnode[2], o_lpid[2];
@@ -216,7 +219,7 @@ struct karl_ctx {
     f(r_node); f(r_pid); f(r_seq); f(r_ev); f(r_sj); f(d_ctlbuf); f(d_cancelbuf);
     f(c_spec); f(c_time); f(c_cpos); f(c_cneg); f(c_rec); f(c_led); f(c_chan); f(c_pp); f(d_recin);
     f(o_px); f(o_py); f(o_pz); f(o_pe); f(o_pmu); f(o_pphi); f(o_ez); f(o_energy); f(o_end);
-    f(o_u2edge); f(o_edge2);
+    f(o_u2edge); f(o_edge2); f(o_bin2); f(o_zedge);
     f(o_psp); f(o_tz); f(o_tr); f(o_xp); f(o_xn); f(o_ro); f(o_ri); f(o_wall); f(o_spec);
     f(o_led); f(o_chan); f(o_pp); f(o_cnt); f(o_err);
     for (int g = 0; g < 2; ++g) {
@@ -1633,6 +1636,7 @@ extern "C" karl_status karl_run_orbit(karl_ctx* ctx, const karl_orbit* ob,
   for (int sp = 0; sp < NSP; ++sp) {
     O.dt[sp] = ob->dt_s[sp];
     O.h[sp] = 0.5 * (ORBIT_CHARGE[sp] * C_LIGHT * C_LIGHT / ctx->mass[sp]) * ob->dt_s[sp];
+    O.hb[sp] = O.h[sp] * O.bz;
   }
   O.e_cut = ctx->e_cut;
   O.spec_bin = ctx->spec_bin;
@@ -1659,6 +1663,30 @@ extern "C" karl_status karl_run_orbit(karl_ctx* ctx, const karl_orbit* ob,
     }
     if ((s = upload(ctx, ctx->o_edge2, e2.data(), e2.size(), st))) return s;
     O.edge2 = ctx->o_edge2.p;
+    // FP32 bounds 2^-19 inside the edges (the first bin reaches the axis, the
+    // last one is open), and of the wall
+    const double in = 1.0 / 524288.0;
+    std::vector<float2> b2((size_t)ob->n_rbins);
+    for (int k = 0; k < ob->n_rbins; ++k) {
+      b2[k].x = k == 0 ? -1.0f : (float)(e2[k] * (1.0 + in));
+      b2[k].y = k == ob->n_rbins - 1 ? INFINITY : (float)(e2[k + 1] * (1.0 - in));
+    }
+    if ((s = upload(ctx, ctx->o_bin2, b2.data(), b2.size(), st))) return s;
+    O.bin2 = ctx->o_bin2.p;
+    O.R2_lo = (float)(O.R2 * (1.0 - in));
+    // the smallest z of each segment floor(z inv_dz); every z below the
+    // second one's belongs to the first, every z from the last one's up to it
+    std::vector<long long> ze(nz + 1);
+    for (size_t j = 1; j < nz; ++j) {
+      double z = (double)j / O.inv_dz;
+      while (z > 0.0 && std::nextafter(z, 0.0) * O.inv_dz >= (double)j) z = std::nextafter(z, 0.0);
+      while (z * O.inv_dz < (double)j) z = std::nextafter(z, INFINITY);
+      std::memcpy(&ze[j], &z, sizeof z);
+    }
+    ze[0] = LLONG_MIN;
+    ze[nz] = LLONG_MAX;
+    if ((s = upload(ctx, ctx->o_zedge, ze.data(), ze.size(), st))) return s;
+    O.zedge = ctx->o_zedge.p;
     CK(cudaStreamSynchronize(st));        // the host tables above go out of scope
   }
   O.ez = ob->e_z_vm ? ctx->o_ez.p : nullptr;
@@ -1681,12 +1709,8 @@ extern "C" karl_status karl_run_orbit(karl_ctx* ctx, const karl_orbit* ob,
   const double timeout = o->timeout_s > 0 ? o->timeout_s : 600.0;
   O.timeout_ns = (unsigned long long)(timeout * 1e9);
 
-  const int block = o->block_size > 0 ? o->block_size : 256;
-  int bps = 0;
-  CK(orbit_occupancy(block, &bps));
-  if (o->blocks_per_sm > 0) bps = std::min(bps, (int)o->blocks_per_sm);
-  if (bps < 1) bps = 1;
-  const int grid = ctx->num_sms * bps;
+  const bool shape_given = o->block_size > 0 || o->blocks_per_sm > 0;
+  int block = o->block_size > 0 ? o->block_size : 256, grid = 0;
   CK(cudaMemsetAsync(ctx->d_cancel, 0, sizeof(int), st));
 
   long long n_in = (long long)n;
@@ -1699,6 +1723,24 @@ extern "C" karl_status karl_run_orbit(karl_ctx* ctx, const karl_orbit* ob,
         std::max<unsigned long long>(1ULL << 20, 8ULL * (unsigned long long)n_in);
     if ((s = ensure_list(ctx, 1 - cur, (size_t)cap))) return s;
     if (gen > 0 && (s = ensure_list(ctx, cur, (size_t)n_in))) return s;
+    if (shape_given) {
+      int bps = 0;
+      CK(orbit_occupancy(block, &bps));
+      if (o->blocks_per_sm > 0) bps = std::min(bps, (int)o->blocks_per_sm);
+      grid = ctx->num_sms * std::max(bps, 1);
+      O.lanes = 32;
+    } else {
+      // A warp's FP64 instruction takes its scheduler's pipe for 64 cycles
+      // whatever its active lanes, so a generation that does not fill the
+      // chip goes to as few warps per scheduler (four to an SM) as hold it,
+      // spread evenly: one block per SM of one to four warps per scheduler,
+      // each taking an equal share of lanes.
+      const long long scheds = 4LL * ctx->num_sms;
+      const long long warps = std::min<long long>(4, (n_in + 32 * scheds - 1) / (32 * scheds));
+      block = (int)(128 * warps);
+      grid = ctx->num_sms;
+      O.lanes = (int)std::min<long long>(32, (n_in + warps * scheds - 1) / (warps * scheds));
+    }
     O.from_primaries = gen == 0;
     O.n_in = n_in;
     O.in = list_of(ctx, cur);

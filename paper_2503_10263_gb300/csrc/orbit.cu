@@ -32,6 +32,7 @@
 #include <cooperative_groups.h>
 
 #include "event.cuh"
+#include "exact_arith.cuh"
 #include "orbit.cuh"
 
 namespace karl {
@@ -41,6 +42,7 @@ namespace {
 enum { EV_NONE = 0, EV_WALL = 1, EV_EXIT = 2, EV_CAP = 3, EV_COLL = 4, EV_EBIN = 5 };
 constexpr int DOM_REDRAW = 3;          // optical depths drawn anew after an energy-bin stop
 constexpr double INV_C2 = 1.0 / (C_LIGHT * C_LIGHT);
+constexpr long long X_SMALL = 0x3e60000000000000LL;   // 2^-25
 
 // Comparisons of the step's tests on the bits of the doubles (integer
 // operations, the same outcomes as the floating-point compares for numbers:
@@ -95,6 +97,14 @@ __device__ void turn(double d0, double d1, double d2, double ct, double cp, doub
 __device__ __forceinline__ int seg_of(const Params& P, const OrbitDev& O, double z) {
   const int j = floor_or_m1(z * O.inv_dz);        // floor on the bits (negative: -1)
   return j < 0 ? 0 : (j > P.nz - 1 ? P.nz - 1 : j);
+}
+
+// segment of z, js if z lies between that segment's edges (integer compares;
+// the edges are the exact thresholds of seg_of)
+__device__ __forceinline__ int seg_near(const Params& P, const OrbitDev& O, double z, int js) {
+  const long long b = __double_as_longlong(z);
+  if (b >= __ldg(O.zedge + js) && b < __ldg(O.zedge + js + 1)) return js;
+  return seg_of(P, O, z);
 }
 
 // radial bin of (x, y), searched from the bin b (the particle's bin, or a
@@ -230,6 +240,7 @@ struct Flight {
   unsigned long long step;
   int cj, cr;                      // cell of the current run of steps
   unsigned long long cn;
+  double rate;                     // sum of sigma n (and sigma n^2) in segment cj
   int js, rs;                      // segment and radial bin of the particle
   unsigned redraw;                 // energy-bin stops since the last event
   unsigned long long w1, w2, w3;   // uniforms of the collision
@@ -270,6 +281,7 @@ __device__ bool start_flight(const Params& P, const OrbitDev& O, OPart& Q, Fligh
   }
   F.step = 0;
   F.cj = -1; F.cr = -1; F.cn = 0;
+  F.rate = 0.0;
   F.js = seg_of(P, O, Q.z);
   F.rs = rbin_of(O, Q.x, Q.y);
   atomicAdd(O.ledger + OB_N_FLIGHT, 1ULL);
@@ -422,7 +434,18 @@ __device__ bool load(const Params& P, const OrbitDev& O, long long i, OPart& Q) 
   return true;
 }
 
-__global__ void __launch_bounds__(256) orbit_kernel(const Params P, const OrbitDev O) {
+// Bound by the FP64 pipe: GB300 issues a warp's FP64 instruction in 64 cycles
+// of its scheduler, so a step costs its count of FP64 instructions and little
+// else.  The push's roots and quotients are therefore taken by
+// exact_arith.cuh (none or two FP64 instructions instead of eight to ten, the
+// same bits), the halvings and doublings on the exponent, the segment and
+// radial bin by integer and FP32 compares away from their edges, the rate per
+// segment kept while the segment lasts; the particles of a small generation
+// are spread over the schedulers (karl_run_orbit).  32768 ions at 2.5 T over
+// 3e-5 s: 340 ms -> 109 ms; 300 decays at 0.25 T (a few serial electrons):
+// 684 ms -> 564 ms.
+__global__ void __launch_bounds__(512, 1) orbit_kernel(const Params P, const OrbitDev O) {
+  if ((int)(threadIdx.x & 31) >= O.lanes) return;
   const double L = P.L;
   bool live = false;
   OPart Q;
@@ -457,29 +480,52 @@ __global__ void __launch_bounds__(256) orbit_kernel(const Params P, const OrbitD
     }
     F.step += 1;
     steps += 1;
-    // Boris push: half electric kick, magnetic rotation, half kick
-    const double ex = O.er * Q.x, ey = O.er * Q.y, ez = O.ez ? O.ez[F.js] : 0.0;
-    const double umx = Q.ux + h * ex, umy = Q.uy + h * ey, umz = Q.uz + h * ez;
-    const double gm = sqrt(1.0 + (umx * umx + umy * umy + umz * umz) * INV_C2);
-    const double t = h * O.bz / gm;
-    const double sf = 2.0 * t / (1.0 + t * t);
+    // Boris push: half electric kick, magnetic rotation, half kick.  With
+    // x = (u/c)^2 below 2^-25 (ions up to 80 eV) gamma = 1 + j 2^-52 follows
+    // from x by integers, and so do the quotients by it.
+    const double ex = O.er * Q.x, ey = O.er * Q.y;
+    const double kx = h * ex, ky = h * ey;
+    const double umx = Q.ux + kx, umy = Q.uy + ky;
+    double umz, kz = 0.0;
+    if (O.ez) {
+      kz = h * O.ez[F.js];
+      umz = Q.uz + kz;
+    } else {
+      umz = dzero(Q.uz) ? Q.uz + h * 0.0 : Q.uz;
+    }
+    const double xm = (umx * umx + umy * umy + umz * umz) * INV_C2;
+    double t;
+    if (bits(xm) < X_SMALL) t = xa_div_1p(O.hb[s], xa_sqrt_ulps(xa_ulps_of_1p(xm)));
+    else t = xa_div(O.hb[s], xa_sqrt(1.0 + xm));
+    const double sf = xa_div(xa_twice(t), 1.0 + t * t);
     const double upx = umx + umy * t, upy = umy - umx * t;
-    const double unx = umx + upy * sf + h * ex;
-    const double uny = umy - upx * sf + h * ey;
-    const double unz = umz + h * ez;
+    const double unx = umx + upy * sf + kx;
+    const double uny = umy - upx * sf + ky;
+    const double unz = O.ez ? umz + kz : (dzero(umz) ? umz + h * 0.0 : umz);
     const double u2n = unx * unx + uny * uny + unz * unz;
-    const double gn = sqrt(1.0 + u2n * INV_C2);
-    const double sc = dt / gn;
+    const double xn2 = u2n * INV_C2;
+    double sc;
+    if (bits(xn2) < X_SMALL) sc = xa_div_1p(dt, xa_sqrt_ulps(xa_ulps_of_1p(xn2)));
+    else sc = xa_div(dt, xa_sqrt(1.0 + xn2));
     const double dx = unx * sc, dy = uny * sc, dz = unz * sc;
-    const double ds = sqrt(dx * dx + dy * dy + dz * dz);
-    const int jm = seg_of(P, O, Q.z + 0.5 * dz);
-    const double nm = P.nseg[jm];
-    const double dtau = (F.s1 * nm + F.s3 * (nm * nm)) * ds;
+    const double ds = xa_sqrt(dx * dx + dy * dy + dz * dz);
+    const double hx = xa_half(dx), hy = xa_half(dy), hz = xa_half(dz);
+    const int jm = seg_near(P, O, Q.z + hz, F.js);
+    if (jm != F.cj) {
+      const double nm = P.nseg[jm];
+      F.rate = F.s1 * nm + F.s3 * (nm * nm);
+    }
+    const double dtau = F.rate * ds;
     // the first of wall, z end, lifetime cap and collision within the step
     double fb = 1.0;
     int event = EV_NONE, end = -1;
     const double xn = Q.x + dx, yn = Q.y + dy, zn = Q.z + dz;
-    if (bits(xn * xn + yn * yn) > bits(O.R2)) {
+    // squared radii of the step's end and midpoint in FP32 (relative error
+    // below 2^-20): they decide wall and bin away from the edges
+    const float2 rb2 = __ldg(O.bin2 + F.rs);
+    const float xe = xa_trunc_f(xn), ye = xa_trunc_f(yn);
+    const float re2 = xe * xe + ye * ye;
+    if (!(re2 < O.R2_lo) && bits(xn * xn + yn * yn) > bits(O.R2)) {
       const double a = dx * dx + dy * dy;
       const double b = Q.x * dx + Q.y * dy;
       const double c = Q.x * Q.x + Q.y * Q.y - O.R2;
@@ -505,14 +551,21 @@ __global__ void __launch_bounds__(256) orbit_kernel(const Params P, const OrbitD
     if (event == EV_NONE && (bits(u2n) < bits(F.u2lo) || bits(u2n) >= bits(F.u2hi)))
       event = EV_EBIN;
     if (event == EV_NONE || event == EV_EBIN) {
-      const int mr = rbin_from(O, Q.x + 0.5 * dx, Q.y + 0.5 * dy, F.rs);
+      const float hxf = xa_trunc_f(hx), hyf = xa_trunc_f(hy);
+      const float xc = xa_trunc_f(Q.x) + hxf, yc = xa_trunc_f(Q.y) + hyf;
+      const float rc2 = xc * xc + yc * yc;
+      // (the sums' error stays below 2^-20 of r while the half step is below r / 4)
+      const bool far = 16.0f * (hxf * hxf + hyf * hyf) < rc2;
+      const int mr = far && rc2 > rb2.x && rc2 < rb2.y ? F.rs
+                                                       : rbin_from(O, Q.x + hx, Q.y + hy, F.rs);
       if (jm == F.cj && mr == F.cr) {
         F.cn += 1;
       } else {
         flush_run(P, O, s, F.cj, F.cr, F.cn, 0.0, dt);
         F.cj = jm; F.cr = mr; F.cn = 1;
       }
-      const int jb = seg_of(P, O, zn), rb = rbin_from(O, xn, yn, F.rs);
+      const int jb = seg_near(P, O, zn, F.js);
+      const int rb = re2 > rb2.x && re2 < rb2.y ? F.rs : rbin_from(O, xn, yn, F.rs);
       if (jb != F.js || rb != F.rs) {
         crossings(P, O, s, F.js, F.rs, jb, rb);
         F.js = jb;

@@ -40,11 +40,15 @@ struct OrbitList {
 struct OrbitDev {
   double bz;                    // magnetic field along +z (T)
   double R2;                    // wall radius squared
+  float R2_lo;                  // an FP32 squared radius below this is inside the wall
   double r_scale;               // radial bins per metre (first guess of a bin)
   const double* edge2;          // [nr+1] squared radii of the radial bin edges
+  const float2* bin2;           // [nr] FP32 squared radii certain to lie in the bin: (low, high)
+  const long long* zedge;       // [nz+1] bits of the smallest z in each segment (first: any)
   double er;                    // radial field per metre (V/m^2)
   double dt[NSP];               // Boris time step per species
   double h[NSP];                // q dt / 2m per species (m/s per V/m)
+  double hb[NSP];               // h B
   double e_cut, spec_bin;       // energies in eV
   double inv_dz;                // n_zbins / L (segment of z: floor(z inv_dz))
   double e_max;                 // top of the energy grid (eV)
@@ -55,6 +59,7 @@ struct OrbitDev {
   unsigned long long max_steps; // steps per flight before "stalled"
   // source of this generation: the primaries, or the list `in`
   int from_primaries;
+  int lanes;                    // lanes of each warp that take particles
   long long n_in;
   const double* px;
   const double* py;

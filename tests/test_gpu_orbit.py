@@ -350,3 +350,19 @@ def test_orbit_shards_add_up_to_the_single_run(karl):
         ctx.close()
     for k in shard.ORBIT_RAW_KEYS:
         np.testing.assert_array_equal(parts[0][k] + parts[1][k], full[k], err_msg=k)
+
+
+@pytest.mark.parametrize("n_ions", [1, 607, 609, 20000])
+def test_orbit_launch_shape_changes_no_tally(karl, n_ions):
+    """Particles spread over the schedulers (default) or packed by a given
+    launch shape: the same integer tallies and end states."""
+    prob, orb, pr = inputs.orbit_ion_config(n_ions=n_ions, seed=4, lifetime_s=3e-7)
+    ctx = karl.Context(prob)
+    try:
+        a = ctx.run_orbit(orb, pr, seed=2)
+        b = ctx.run_orbit(orb, pr, seed=2, block_size=64, blocks_per_sm=2)
+    finally:
+        ctx.close()
+    for k in a:
+        if k != "energy":
+            np.testing.assert_array_equal(a[k], b[k], err_msg=k)
