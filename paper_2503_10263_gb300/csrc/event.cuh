@@ -297,9 +297,6 @@ __device__ __forceinline__ void emit(RingPort& port, const Lane& p) {
       port.q->s[i] = p;
       placed = true;
     }
-    const int kept = base >= WQ ? 0 : min(WQ - base, n);
-    if (!port.slot_live && g.thread_rank() == 0 && kept > 0)
-      atomicAdd((unsigned long long*)&port.ctl->active, (unsigned long long)kept);  // held by this warp
   }
   if (!placed) {
     cg::coalesced_group g = cg::coalesced_threads();

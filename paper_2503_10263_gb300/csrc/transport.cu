@@ -7,8 +7,9 @@
 // segment-stop mover of Sec. 3.1), the time/density and current tallies of
 // Secs. 2.2-2.3 as range adds, the terminator of Sec. 3.2, a channel chosen
 // with probability sigma_i n_i / sum_j sigma_j n_j, and its kinematics
-// (Sec. 3.3).  Products go to a device-wide ring; lanes whose particle ended
-// take the next one from the ring (products first) or from the primaries.
+// (Sec. 3.3).  Products go to their warp's queue and, past its end or when
+// lanes elsewhere are idle, to a device-wide ring; lanes whose particle ended
+// take the next one from their queue, from the ring or from the primaries.
 // All waits are bounded by iteration counts and a wall-clock deadline, after
 // which the kernel records an error and returns.
 #include "event.cuh"
@@ -17,6 +18,10 @@ namespace karl {
 
 // ---------------------------------------------------------------------------
 // persistent kernel
+
+// Particles of a warp's queue that a claim on the ring may fill (half the
+// queue, so the products of the next events still find room).
+constexpr int RING_BATCH = WQ / 2;
 
 // Copy the column tables (and the pass-2 recombination fields) into dynamic
 // shared memory when they fit; the event code reads them through P's pointers.
@@ -89,7 +94,7 @@ __global__ void __launch_bounds__(512, 1) transport_kernel(const Params Pk, Ring
   const unsigned lt = (1u << lane) - 1u;
   WarpQueue& Q = wq[threadIdx.x >> 5];
   RareBuf& Rb = rbuf[threadIdx.x >> 5];
-  bool eager = false;
+  const int wid = threadIdx.x >> 5;
   bool has = false;
   Lane L;
   EventOut o;
@@ -117,10 +122,40 @@ __global__ void __launch_bounds__(512, 1) transport_kernel(const Params Pk, Ring
   port.spilled = 0;
   port.slot_live = nullptr;
 
+  // ctl->active counts the particles the warps hold (lanes, queues, parked
+  // collisions) plus each warp's `credit`: places counted there that hold
+  // nothing now.  Deaths raise the credit, refills and products use it up
+  // before they add to the counter, and what is left is returned at the next
+  // look at the counters, so most deaths and refills take no global atomic.
+  int credit = 0;
+  // Warps of a block that take part, in steps of four (warp w of a block runs
+  // on scheduler w mod 4).  A warp's FP64 instruction takes its scheduler's
+  // pipe for 64 cycles whatever its active lanes, so particles that do not
+  // fill the chip go to as few warps per scheduler as hold them: a run of few
+  // primaries starts with an equal share (`quota`) on every participating
+  // warp, and once the primaries are used up the warps from T on hand their
+  // particles to the shared ring, where those below T take them.  T follows
+  // the number of particles alive: up when 95 % of the places of the warps
+  // below it are taken, down when the particles fill 70 % of the next fewer.
+  // Measured with the claims of up to RING_BATCH below, pass 1 of the source
+  // run: 1e5 decays FP64 144.8 -> 73 ms, FP32 108 -> 41 ms, 1e6 decays FP64
+  // 524 -> 484 ms, 1e3 decays FP64 13.0 -> 8.5 ms.
+  const long long step_lanes = 128LL * gridDim.x;
+  int T = 4;
+  while (T < nwarps && step_lanes * (T >> 2) < P.n_prim) T += 4;
+  const long long first_warps = (long long)gridDim.x * min(T, nwarps);
+  const int quota = (int)min(32LL, (P.n_prim + first_warps - 1) / first_warps);
+  bool drained = false;       // every primary is claimed
+  bool share = false;         // idle lanes elsewhere: surplus products go to the ring
+  bool eager = false;         // parked collisions go at once
+  bool idle = false;          // the last iteration found no particle
+
   for (long long iter = 0;; ++iter) {
-    if ((iter & 63) == 0) {
-      int stop = 0;
+    if ((iter & 15) == 0 || idle) {
+      // lane 0 reads the counters and decides for the warp
+      int word = 0;
       if (lane == 0) {
+        int stop = 0;
         if (ld_relaxed_i(&ctl->abort)) stop = 1;
         else if (cancel && ld_relaxed_i((const int*)cancel)) {
           atomicCAS(&ctl->error, 0, ERR_CANCELLED);
@@ -131,18 +166,69 @@ __global__ void __launch_bounds__(512, 1) transport_kernel(const Params Pk, Ring
           atomicExch(&ctl->abort, 1);
           stop = 1;
         }
+        const unsigned long long h = ld_relaxed(&ctl->head), t = ld_relaxed(&ctl->tail);
+        const long long pn = (long long)ld_relaxed(&ctl->prim_next);
+        const long long act = ld_relaxed_s(&ctl->active);
+        const long long left = max(0LL, P.n_prim - pn);
+        const long long alive = max(0LL, act - credit) + (t > h ? (long long)(t - h) : 0LL) + left;
+        int n = T;
+        while (n < nwarps && alive * 20 > step_lanes * (n >> 2) * 19) n += 4;
+        while (n > 4 && alive * 10 < step_lanes * ((n >> 2) - 1) * 7) n -= 4;
+        const int dr = left == 0;
+        const int sh = dr && t - h < (unsigned long long)step_lanes &&
+                       alive * 50 < 32LL * gridDim.x * nwarps * 49;
+        // The last primaries' histories set the end of the pass: from about
+        // two primaries per lane before the end, parked collisions go at once
+        // so those histories are not held up.
+        const int eg = left <= 2LL * gridDim.x * blockDim.x;
+        word = stop | (dr << 1) | (sh << 2) | (eg << 3) | (t > h ? 16 : 0) | (n << 8);
+        if (credit > 0) {
+          __threadfence();
+          atomicAdd((unsigned long long*)&ctl->active, (unsigned long long)(-(long long)credit));
+        }
       }
-      if (__shfl_sync(FULL, stop, 0)) break;
-      const unsigned long long pn = ld_relaxed(&ctl->prim_next);
-      port.local = pn < (unsigned long long)P.n_prim;
-      // The last primaries' histories set the end of the pass: from about two
-      // primaries per lane before the end, parked collisions go at once so
-      // those histories are not held up.
-      eager = pn + 2ULL * gridDim.x * blockDim.x >= (unsigned long long)P.n_prim;
+      credit = 0;
+      word = __shfl_sync(FULL, word, 0);
+      if (word & 1) break;
+      drained = (word & 2) != 0;
+      share = (word & 4) != 0;
+      eager = (word & 8) != 0;
+      if (word & 16) refill_skip = 0;             // the ring has work
+      T = word >> 8;
+    }
+    const bool serves = wid < T;
+
+    // ---- warps from T on hand what they hold to the ring ----
+    __syncwarp();
+    if (!serves && drained) {
+      const unsigned m = __ballot_sync(FULL, has);
+      const int k = __popc(m), q = min(Q.top, WQ), r = Rb.r, tot = k + q + r;
+      if (tot > 0) {
+        unsigned long long pos = 0;
+        if (lane == 0) pos = atomicAdd(&ctl->tail, (unsigned long long)tot);
+        pos = __shfl_sync(FULL, pos, 0);
+        if (has) {
+          ring_put(R, ctl, pos + __popc(m & lt), L, deadline);
+          started -= 1;                           // counted again when taken
+          has = false;
+        }
+        if (lane < q) ring_put(R, ctl, pos + k + lane, Q.s[lane], deadline);
+        if (lane < r) {
+          ring_put(R, ctl, pos + k + q + lane, Rb.s[RB - r + lane], deadline);
+          started -= 1;
+        }
+        __syncwarp();
+        if (lane == 0) {
+          Q.top = 0;
+          Rb.r = 0;
+          port.spilled += tot;
+        }
+        credit += tot;
+        __syncwarp();
+      }
     }
 
     // ---- idle lanes first resume particles handed back for a batch ----
-    __syncwarp();
     if (Rb.r > 0) {
       const unsigned needr = __ballot_sync(FULL, !has);
       const int r0 = Rb.r;
@@ -160,11 +246,10 @@ __global__ void __launch_bounds__(512, 1) transport_kernel(const Params Pk, Ring
     }
 
     // ---- idle lanes take the warp's own products first (newest first) ----
-    __syncwarp();
+    int qleft;                                    // products left in the queue
     {
       const unsigned need0 = __ballot_sync(FULL, !has);
-      int top = Q.top;
-      if (top > WQ) top = WQ;
+      const int top = Q.top;
       const int take = min(__popc(need0), top);
       if (!has) {
         const int rank = __popc(need0 & lt);
@@ -174,29 +259,24 @@ __global__ void __launch_bounds__(512, 1) transport_kernel(const Params Pk, Ring
           started += 1;
         }
       }
-      int left = top - take;
-      // once the primaries are used up, move what is left to the shared ring
-      // where idle warps can take it (counted there instead of here)
-      if (!port.local && left > 0) {
+      qleft = top - take;
+      // surplus products go to the shared ring while lanes elsewhere are idle
+      if (share && qleft > 0) {
         unsigned long long pos = 0;
-        if (lane == 0) pos = atomicAdd(&ctl->tail, (unsigned long long)left);
+        if (lane == 0) pos = atomicAdd(&ctl->tail, (unsigned long long)qleft);
         pos = __shfl_sync(FULL, pos, 0);
-        if (lane < left) ring_put(R, ctl, pos + lane, Q.s[lane], deadline);
-        __syncwarp();
-        if (lane == 0) {
-          __threadfence();
-          atomicAdd((unsigned long long*)&ctl->active, (unsigned long long)(-(long long)left));
-          port.spilled += left;
-        }
-        left = 0;
+        if (lane < qleft) ring_put(R, ctl, pos + lane, Q.s[lane], deadline);
+        if (lane == 0) port.spilled += qleft;
+        credit += qleft;
+        qleft = 0;
       }
       __syncwarp();
-      if (lane == 0) Q.top = left;
+      if (lane == 0) Q.top = qleft;
       __syncwarp();
     }
 
     // ---- other idle lanes take work: products from the ring, then primaries ----
-    unsigned need = __ballot_sync(FULL, !has);
+    unsigned need = serves ? __ballot_sync(FULL, !has) : 0u;
     if (need && need != FULL && refill_skip > 0) {
       --refill_skip;
       need = 0;
@@ -204,7 +284,12 @@ __global__ void __launch_bounds__(512, 1) transport_kernel(const Params Pk, Ring
     if (need) {
       const int k = __popc(need);
       unsigned long long rbase = 0, pbase = 0;
-      int rgot = 0, pgot = 0;
+      int rgot = 0, pgot = 0, cr = credit;
+      // With a long ring a warp takes up to half its even share of it in one
+      // claim: what its lanes have no room for waits in its queue.  (One
+      // claim per few particles held the whole chip to about 11 particles a
+      // microsecond, a fifth of what 75-event histories use up.)
+      const int spare = max(0, RING_BATCH - qleft);
       if (lane == 0) {
         // Count the lanes as active only when work is visible, then claim it:
         // idle warps that find nothing leave the counter alone.  Lanes the
@@ -214,37 +299,50 @@ __global__ void __launch_bounds__(512, 1) transport_kernel(const Params Pk, Ring
         // lanes back for a ring only a quarter full left a quarter of the
         // FP32 form's lanes idle while every warp fought for the ring head.
         unsigned long long h = ld_relaxed(&ctl->head), t = ld_relaxed(&ctl->tail);
-        const unsigned long long pn = ld_relaxed(&ctl->prim_next);
-        const bool ring_work = h < t;
-        const bool prim_work = pn < (unsigned long long)P.n_prim && t - h < R.cap / 4 * 3;
-        if (ring_work || prim_work) {
-          atomicAdd((unsigned long long*)&ctl->active, (unsigned long long)k);
-          __threadfence();
+        const unsigned long long pn = drained ? (unsigned long long)P.n_prim
+                                              : ld_relaxed(&ctl->prim_next);
+        const int room = max(0, quota - (32 - k));          // primaries this warp may take
+        const bool prim_work = pn < (unsigned long long)P.n_prim && room > 0 &&
+                               (h >= t || t - h < R.cap / 4 * 3);
+        const unsigned long long ready = h < t ? t - h : 0ULL;
+        const unsigned long long fair = ready / (2ULL * gridDim.x * nwarps);
+        const int extra = fair <= (unsigned long long)k
+                              ? 0
+                              : (fair - k < (unsigned long long)spare ? (int)(fair - k) : spare);
+        const unsigned long long all = ready + (prim_work ? room : 0);
+        const int want = all < (unsigned long long)(k + extra) ? (int)all : k + extra;
+        if (want > 0) {
+          if (cr < want) {
+            atomicAdd((unsigned long long*)&ctl->active, (unsigned long long)(want - cr));
+            __threadfence();
+            cr = want;
+          }
           for (int tries = 0; tries < 16 && h < t; ++tries) {
-            unsigned long long take = t - h < (unsigned long long)k ? t - h : (unsigned long long)k;
+            unsigned long long take =
+                t - h < (unsigned long long)want ? t - h : (unsigned long long)want;
             unsigned long long old = atomicCAS(&ctl->head, h, h + take);
             if (old == h) { rbase = h; rgot = (int)take; break; }
             h = old;
             t = ld_relaxed(&ctl->tail);
           }
-          if (rgot < k && prim_work) {
-            const int want = k - rgot;
-            unsigned long long p0 = atomicAdd(&ctl->prim_next, (unsigned long long)want);
+          const int wp = min(min(want, k) - rgot, room);
+          if (wp > 0 && prim_work) {
+            unsigned long long p0 = atomicAdd(&ctl->prim_next, (unsigned long long)wp);
             if (p0 < (unsigned long long)P.n_prim) {
               unsigned long long left = (unsigned long long)P.n_prim - p0;
               pbase = p0;
-              pgot = left < (unsigned long long)want ? (int)left : want;
-              if (left <= (unsigned long long)want) atomicMax(&ctl->t_claimed, globaltimer_ns());
+              pgot = left < (unsigned long long)wp ? (int)left : wp;
+              if (left <= (unsigned long long)wp) atomicMax(&ctl->t_claimed, globaltimer_ns());
             }
           }
-          if (rgot + pgot < k)
-            atomicAdd((unsigned long long*)&ctl->active, (unsigned long long)(rgot + pgot - k));
+          cr -= rgot + pgot;
         }
       }
       rbase = __shfl_sync(FULL, rbase, 0);
       pbase = __shfl_sync(FULL, pbase, 0);
       rgot = __shfl_sync(FULL, rgot, 0);
       pgot = __shfl_sync(FULL, pgot, 0);
+      credit = __shfl_sync(FULL, cr, 0);
       if (rgot + pgot == 0) {
         refill_backoff = refill_backoff * 2 + 1;
         if (refill_backoff > 63) refill_backoff = 63;
@@ -282,10 +380,14 @@ __global__ void __launch_bounds__(512, 1) transport_kernel(const Params Pk, Ring
           started += 1;
         }
       }
-      const unsigned md = __ballot_sync(FULL, born_dead);
-      if (md && lane == 0) {
-        __threadfence();
-        atomicAdd((unsigned long long*)&ctl->active, (unsigned long long)(-(long long)__popc(md)));
+      credit += __popc(__ballot_sync(FULL, born_dead));
+      if (rgot > k) {                              // more than the idle lanes: to the queue
+        const int more = rgot - k;
+        if (lane < more) ring_get(R, ctl, rbase + k + lane, Q.s[qleft + lane], deadline);
+        qleft += more;
+        __syncwarp();
+        if (lane == 0) Q.top = qleft;
+        __syncwarp();
       }
     }
 
@@ -323,9 +425,14 @@ __global__ void __launch_bounds__(512, 1) transport_kernel(const Params Pk, Ring
     }
 
     const unsigned busy = __ballot_sync(FULL, has);
-    if (!busy) {
+    idle = !busy;
+    if (idle) {
       int done = 0;
       if (lane == 0) {
+        if (credit > 0) {
+          __threadfence();
+          atomicAdd((unsigned long long*)&ctl->active, (unsigned long long)(-(long long)credit));
+        }
         // Done when no work is queued, none will come (no particle is held),
         // and nothing moved between two snapshots taken around the read of
         // the active count.  A claim visible in the first snapshot makes its
@@ -341,6 +448,7 @@ __global__ void __launch_bounds__(512, 1) transport_kernel(const Params Pk, Ring
         done = (a <= 0 && h1 == h2 && t1 == t2 && p1 == p2 && h1 >= t1 &&
                 p1 >= (unsigned long long)P.n_prim);
       }
+      credit = 0;
       if (__shfl_sync(FULL, done, 0)) break;
       __nanosleep(idle_ns);
       if (idle_ns < 4096) idle_ns <<= 1;
@@ -366,8 +474,10 @@ __global__ void __launch_bounds__(512, 1) transport_kernel(const Params Pk, Ring
       if (!o.alive) { has = false; died = !o.parked; }
     }
     __syncwarp();
+    const int qtop = min(Q.top, WQ);                  // pushes past the end went to the ring
+    __syncwarp();
     if (lane == 0) {
-      if (Q.top > WQ) Q.top = WQ;                     // pushes past the end went to the ring
+      Q.top = qtop;
       if (Rb.n > RB - Rb.r) Rb.n = RB - Rb.r;         // parks past the end were done in line
     }
 
@@ -379,11 +489,11 @@ __global__ void __launch_bounds__(512, 1) transport_kernel(const Params Pk, Ring
     }
     o.chan = -1;
 
-    const unsigned md = __ballot_sync(FULL, died);
-    if (md) {
-      __threadfence();
+    credit += __popc(__ballot_sync(FULL, died)) - (qtop - qleft);
+    if (credit < 0) {                                 // more products than places
       if (lane == 0)
-        atomicAdd((unsigned long long*)&ctl->active, (unsigned long long)(-(long long)__popc(md)));
+        atomicAdd((unsigned long long*)&ctl->active, (unsigned long long)(-(long long)credit));
+      credit = 0;
     }
   }
 
