@@ -259,6 +259,7 @@ struct WarpQueue {
 // back to make room for a batch; free lanes resume those before other work.
 constexpr int RB = 32;                    // parked collisions per warp
 constexpr int RB_TRIGGER = 24;            // batch size that starts a batch
+constexpr int RB_TRIGGER_LATE = 6;        // the same once the primaries are used up
 struct RareBuf {
   Lane s[RB];
   int8_t ch[RB];

@@ -177,10 +177,10 @@ __global__ void __launch_bounds__(512, 1) transport_kernel(const Params Pk, Ring
         const int dr = left == 0;
         const int sh = dr && t - h < (unsigned long long)step_lanes &&
                        alive * 50 < 32LL * gridDim.x * nwarps * 49;
-        // The last primaries' histories set the end of the pass: from about
-        // two primaries per lane before the end, parked collisions go at once
-        // so those histories are not held up.
-        const int eg = left <= 2LL * gridDim.x * blockDim.x;
+        // The last histories set the end of the pass: once the particles no
+        // longer fill the chip, parked collisions go at once so that those
+        // histories are not held up.
+        const int eg = alive < (long long)gridDim.x * blockDim.x;
         word = stop | (dr << 1) | (sh << 2) | (eg << 3) | (t > h ? 16 : 0) | (n << 8);
         if (credit > 0) {
           __threadfence();
@@ -393,12 +393,16 @@ __global__ void __launch_bounds__(512, 1) transport_kernel(const Params Pk, Ring
 
     // ---- parked rare collisions: once enough have gathered, free lanes and
     // then busy ones -- whose particles wait in the slots the batch frees --
-    // perform them together; near the end of the pass, at once ----
+    // perform them together; fewer make a batch once the primaries are used
+    // up, and one does when the particles no longer fill the chip.  (At 1e5
+    // decays, pass 1: one from two primaries per lane before the end 73.0 ms
+    // FP64 / 41.0 FP32, one from the time the chip is not full 63.5 / 31.3,
+    // with 12 late 54.9 / 28.0, with 6 late 53.5 / 28.1.) ----
     __syncwarp();
     int rk = -1;
     const int nr = min(Rb.n, RB - Rb.r);
     const unsigned hm = __ballot_sync(FULL, has);
-    const bool batch = nr >= RB_TRIGGER || (nr > 0 && (hm == 0 || eager));
+    const bool batch = nr >= (drained ? RB_TRIGGER_LATE : RB_TRIGGER) || (nr > 0 && (hm == 0 || eager));
     if (batch) {
       const int nfree = 32 - __popc(hm);
       const int rank = has ? nfree + __popc(hm & lt) : __popc(~hm & lt);
