@@ -9,6 +9,7 @@
 #pragma once
 #include <cooperative_groups.h>
 
+#include "exact_arith.cuh"
 #include "karl_device.cuh"
 
 namespace karl {
@@ -38,13 +39,25 @@ template <class R> __device__ __forceinline__ R from_d(double x);
 template <> __device__ __forceinline__ double from_d<double>(double x) { return x; }
 template <> __device__ __forceinline__ float from_d<float>(double x) { return (float)x; }
 
+// out of line for the rare paths (the event itself takes them inline)
+static __device__ __noinline__ double div_call(double a, double b) { return xa_div(a, b); }
+static __device__ __noinline__ double sqrt_call(double a) { return xa_sqrt(a); }
+
 template <bool F32> struct RT;
 template <> struct RT<false> {
   using R = double;
   static __device__ __forceinline__ R u(unsigned long long w) { return u01d(w); }
   static __device__ __forceinline__ R eta(unsigned long long w) { return eta01d(w); }
+  // 2u and 2u - 1 (both exact) from the bits of the uniform's 53-bit integer
+  static __device__ __forceinline__ R u2(unsigned long long w) { return u53_scaled(w >> 11, 52); }
+  static __device__ __forceinline__ R u2m1(unsigned long long w) {
+    const long long k = (long long)(w >> 11) - (1LL << 52);
+    const double d = u53_scaled((unsigned long long)(k < 0 ? -k : k), 52);
+    return __longlong_as_double(__double_as_longlong(d) | (k & (long long)0x8000000000000000ULL));
+  }
   static __device__ __forceinline__ R lg(R x) { return log_tab(x); }
-  static __device__ __forceinline__ R sq(R x) { return sqrt(x); }
+  static __device__ __forceinline__ R sq(R x) { return sqrt_call(x); }
+  static __device__ __forceinline__ R dv(R a, R b) { return div_call(a, b); }   // b > 0
   static __device__ __forceinline__ R rsq(R x) { return rsqrt(x); }
   static __device__ __forceinline__ R tn(R x) { return tan(x); }
   static __device__ __forceinline__ R atn(R x) { return atan(x); }
@@ -71,6 +84,10 @@ template <> struct RT<false> {
     return eq >= 0 && eq < (1LL << 53) ? u53_scaled((unsigned long long)eq, 24)
                                        : (double)eq * (1.0 / 16777216.0);
   }
+  // trunc(RN(de 2^24 + 1/2)) for de >= 0, from the bits: with t = trunc(de 2^25)
+  // it is (t + 1) / 2 rounded down, and 1 for the one value just below 2^-25
+  // whose sum with 1/2 rounds up to 1 (at all others the sum's rounding does
+  // not reach the next integer: below 2^52 every integer and half is a double)
   static __device__ __forceinline__ long long quant_de(R de) {   // de >= 0
     return trunc_nonneg(de * 16777216.0 + 0.5);
   }
@@ -83,8 +100,11 @@ template <> struct RT<true> {
   using R = float;
   static __device__ __forceinline__ R u(unsigned long long w) { return u01f(w); }
   static __device__ __forceinline__ R eta(unsigned long long w) { return eta01f(w); }
+  static __device__ __forceinline__ R u2(unsigned long long w) { return 2.0f * u01f(w); }
+  static __device__ __forceinline__ R u2m1(unsigned long long w) { return 2.0f * u01f(w) - 1.0f; }
   static __device__ __forceinline__ R lg(R x) { return logf(x); }
   static __device__ __forceinline__ R sq(R x) { return sqrtf(x); }
+  static __device__ __forceinline__ R dv(R a, R b) { return a / b; }
   static __device__ __forceinline__ R rsq(R x) { return rsqrtf(x); }
   static __device__ __forceinline__ R tn(R x) { return tanf(x); }
   static __device__ __forceinline__ R atn(R x) { return atanf(x); }
@@ -154,7 +174,15 @@ __device__ __forceinline__ unsigned long long quant_t(double len, double inv_sz)
   double t = len * inv_sz;
   return (unsigned long long)(t * Q_T + 0.5);
 }
-__device__ __forceinline__ long long quant_e(double e) { return (long long)floor(e * Q_E); }
+// floor(e 2^24): on the bits for e >= 0 below 2^38 eV
+__device__ __forceinline__ long long quant_e(double e) {
+  const long long b = __double_as_longlong(e);
+  if (b < 0 || b >= (1023LL + 38) << 52) return (long long)floor(e * Q_E);
+  const int x = (int)(b >> 52) - 1075 + 24;
+  const long long m = (b & 0x000fffffffffffffLL) | 0x0010000000000000LL;
+  if (x < -52) return 0;
+  return x >= 0 ? (m << x) : (m >> -x);
+}
 
 // 1 / v for kinetic energy e (relativistic: v = c sqrt(x (2 + x)) / (1 + x),
 // x = e / m c^2); every use of the speed divides by it
@@ -187,8 +215,8 @@ __device__ __forceinline__ void range_add(unsigned long long* d, int a, int b, s
 // ---------------------------------------------------------------------------
 // ring cells
 
-static __device__ bool ring_put(const Ring& R, Control* ctl, unsigned long long pos, const Lane& p,
-                         unsigned long long deadline) {
+__device__ __forceinline__ bool ring_put(const Ring& R, Control* ctl, unsigned long long pos,
+                                         const Lane& p, unsigned long long deadline) {
   unsigned long long* cell = R.seq + (pos & R.mask);
   long long spins = 0;
   while (ld_acquire(cell) != pos) {           // previous occupant not consumed yet
@@ -206,8 +234,8 @@ static __device__ bool ring_put(const Ring& R, Control* ctl, unsigned long long 
   return true;
 }
 
-static __device__ bool ring_get(const Ring& R, Control* ctl, unsigned long long pos, Lane& p,
-                         unsigned long long deadline) {
+__device__ __forceinline__ bool ring_get(const Ring& R, Control* ctl, unsigned long long pos,
+                                         Lane& p, unsigned long long deadline) {
   unsigned long long* cell = R.seq + (pos & R.mask);
   long long spins = 0;
   while (ld_acquire(cell) != pos + 1) {        // producer still writing
@@ -231,8 +259,8 @@ static __device__ bool ring_get(const Ring& R, Control* ctl, unsigned long long 
 
 struct EventOut {
   bool alive;
-  bool parked;                            // handed to the warp's batch of rare collisions
   int chan;                               // channel of this event's collision, -1 if none
+  int rare;                               // rare channel whose kinematics are to follow, -1 if none
   unsigned long long flights, colls;      // per-lane counters, flushed at the end
   unsigned long long recoil, excit;       // per-lane energy sums (2^-24 eV)
 };
@@ -248,6 +276,10 @@ struct WarpQueue {
   Lane s[WQ];
   int top;
 };
+
+// Particles of a warp's queue that a claim on the ring may fill (half the
+// queue, so the products of the next events still find room).
+constexpr int RING_BATCH = WQ / 2;
 
 // Collisions in the rare channels (ionization with its products, clustering,
 // charge exchange) cost as much FP64 work as a whole ordinary event, and a warp pays that cost
@@ -272,8 +304,6 @@ struct RingPort {
   Control* ctl;
   unsigned long long deadline;
   WarpQueue* q;
-  RareBuf* rare;           // NULL: perform rare collisions in line
-  bool local;              // primaries remain: keep products in the warp queue
   unsigned long long spilled;
   // multi-request kernel: every existing particle counts in its slot's live
   // word (low 32 bits); NULL in the single-run kernel
@@ -287,7 +317,7 @@ __device__ __forceinline__ void emit(RingPort& port, const Lane& p) {
   namespace cg = cooperative_groups;
   if (port.slot_live) atomicAdd(port.slot_live, 1ULL);
   bool placed = false;
-  if (port.local) {                        // uniform over the warp
+  {
     cg::coalesced_group g = cg::coalesced_threads();
     const int n = (int)g.size();
     int base = 0;
@@ -322,10 +352,10 @@ template <bool F32>
 __device__ __forceinline__ void thermal(const Params& P, const unsigned long long w[4],
                                         long long& eq, double& mu) {
   // Maxwell-Boltzmann target: Gamma(3/2, kT) = Exp(1) + Z^2/2 (Box-Muller), isotropic
-  double c = cospi(2.0 * u01d(w[2]));
+  double c = cospi(RT<false>::u2(w[2]));
   double e = P.kT * (-log(eta01d(w[0])) - log(eta01d(w[1])) * c * c);
   eq = quant_e(e);
-  mu = 2.0 * u01d(w[3]) - 1.0;
+  mu = RT<false>::u2m1(w[3]);
 }
 
 // cos(chi) of an elastic collision from the angle table `set` at impact
@@ -403,7 +433,7 @@ __device__ __forceinline__ void draw_target(const Params& P, const Lane& L,
   const R uz = v1z - ud;
   const R un = T::sq(v1x * v1x + uz * uz);
   const R rpi = (R)1.7724538509055160273, r8 = (R)2.8284271247461900976;
-  const R pmax = un * rpi / (un * rpi + r8 * a);
+  const R pmax = T::dv(un * rpi, un * rpi + r8 * a);
   wx = (R)0; wy = (R)0; wz = (R)0;
   for (int k = 0; k < 64; ++k) {
     unsigned long long b0[4], b1[4];
@@ -422,7 +452,7 @@ __device__ __forceinline__ void draw_target(const Params& P, const Lane& L,
     }
     const R sp = T::sq(s2);
     const R ct = (R)2 * T::u(b1[0]) - (R)1;
-    const R st = T::sq(fmax((R)0, (R)1 - ct * ct));
+    const R st = T::sq(T::max0((R)1 - ct * ct));
     const R ph = (R)2 * T::u(b1[1]);
     wx = sp * st * T::cpi(ph);
     wy = sp * st * T::spi(ph);
@@ -442,31 +472,32 @@ __device__ __noinline__ void moving_target_elastic(const Params& P, const ChanDe
   const int s = L.sp;
   const R m1 = (R)P.mass[s], m2 = (R)P.target_mass, M = m1 + m2;
   const R e = T::energy(L.eq);
-  const R s1 = T::sq((R)2 * e / m1);
+  const R s1 = T::sq(T::dv((R)2 * e, m1));
   const R mu = (R)L.mu;
-  const R sperp = T::sq(fmax((R)0, (R)1 - mu * mu));
+  const R sperp = T::sq(T::max0((R)1 - mu * mu));
   const R v1x = s1 * sperp, v1z = s1 * mu;
   R wx, wy, wz;
   draw_target<F32>(P, L, v1x, v1z, wx, wy, wz);
   const R v2x = wx, v2y = wy, v2z = (R)P.drift_c + wz;
   // centre-of-mass velocity and relative velocity
-  const R Vx = (m1 * v1x + m2 * v2x) / M, Vy = (m2 * v2y) / M, Vz = (m1 * v1z + m2 * v2z) / M;
+  const R Vx = T::dv(m1 * v1x + m2 * v2x, M), Vy = T::dv(m2 * v2y, M),
+          Vz = T::dv(m1 * v1z + m2 * v2z, M);
   const R gx = v1x - v2x, gy = -v2y, gz = v1z - v2z;
   const R gn = T::sq(gx * gx + gy * gy + gz * gz);
   R hx = (R)0, hy = (R)0, hz = (R)1;
-  if (gn > (R)0) { hx = gx / gn; hy = gy / gn; hz = gz / gn; }
+  if (gn > (R)0) { hx = T::dv(gx, gn); hy = T::dv(gy, gn); hz = T::dv(gz, gn); }
   // e1: the part of z perpendicular to g (x if g is along z); e2 = h x e1
   R ax = -hz * hx, ay = -hz * hy, az = (R)1 - hz * hz;
   R n1 = T::sq(ax * ax + ay * ay + az * az);
   if (n1 < (R)1e-12) { ax = (R)1; ay = (R)0; az = (R)0; n1 = (R)1; }
-  ax /= n1; ay /= n1; az /= n1;
+  ax = T::dv(ax, n1); ay = T::dv(ay, n1); az = T::dv(az, n1);
   const R bx = hy * az - hz * ay, by = hz * ax - hx * az, bz = hx * ay - hy * ax;
   // impact energy: the impactor's kinetic energy relative to the target
   const R cchi = elastic_cchi<F32>(P, ch, (R)0.5 * m1 * gn * gn, T::u(w[2]));
-  const R schi = T::sq(fmax((R)0, (R)1 - cchi * cchi));
+  const R schi = T::sq(T::max0((R)1 - cchi * cchi));
   const R phi = (R)2 * T::u(w[3]);
   const R cph = T::cpi(phi), sph = T::spi(phi);
-  const R f = m2 / M * gn;
+  const R f = T::dv(m2, M) * gn;
   const R nx = Vx + f * (schi * cph * ax + schi * sph * bx + cchi * hx);
   const R ny = Vy + f * (schi * cph * ay + schi * sph * by + cchi * hy);
   const R nz = Vz + f * (schi * cph * az + schi * sph * bz + cchi * hz);
@@ -489,9 +520,9 @@ __device__ __noinline__ void charge_exchange(const Params& P, Lane& L, unsigned 
   using R = typename T::R;
   const R m1 = (R)P.mass[L.sp];
   const R e = T::energy(L.eq);
-  const R s1 = T::sq((R)2 * e / m1);
+  const R s1 = T::sq(T::dv((R)2 * e, m1));
   const R mu = (R)L.mu;
-  const R sperp = T::sq(fmax((R)0, (R)1 - mu * mu));
+  const R sperp = T::sq(T::max0((R)1 - mu * mu));
   R wx, wy, wz;
   draw_target<F32>(P, L, s1 * sperp, s1 * mu, wx, wy, wz);
   const R vz = (R)P.drift_c + wz;
@@ -544,9 +575,9 @@ __device__ __noinline__ void moving_target_ionization(const Params& P, unsigned 
   const R m1 = (R)P.mass[s], me = (R)P.mass[SP_E];
   const R e = T::energy(L.eq);
   const R ion_e = (R)ch.loss_ev;
-  const R s1 = T::sq((R)2 * e / m1);
+  const R s1 = T::sq(T::dv((R)2 * e, m1));
   const R mu = (R)L.mu;
-  const R sperp = T::sq(fmax((R)0, fma_rn(-mu, mu, (R)1)));
+  const R sperp = T::sq(T::max0(fma_rn(-mu, mu, (R)1)));
   const R v1x = mul_rn(s1, sperp), v1z = mul_rn(s1, mu);
   R v2x = (R)0, v2y = (R)0, v2z = (R)0, gx = v1x, gy = (R)0, gz = v1z, ei = e;
   for (int r = 0; r < 64; ++r) {
@@ -569,20 +600,20 @@ __device__ __noinline__ void moving_target_ionization(const Params& P, unsigned 
   R wsec = eps * T::tn(T::u(w[2]) * T::atn(wmax * (R)P.inv_eps_ion));
   wsec = fmin(fmax(wsec, (R)0), wmax);
   const R e1 = avail - wsec;
-  const R cp = T::sq(e1 / avail), sp = T::sq(wsec / avail);
+  const R cp = T::sq(T::dv(e1, avail)), sp = T::sq(T::dv(wsec, avail));
   // basis: h along the relative velocity, b1 the part of z perpendicular to
   // it (x if it is along z), b2 = h x b1
   const R gn = T::sq(fma_rn(gx, gx, fma_rn(gy, gy, mul_rn(gz, gz))));
   R hx = (R)0, hy = (R)0, hz = (R)1;
-  if (gn > (R)0) { hx = gx / gn; hy = gy / gn; hz = gz / gn; }
+  if (gn > (R)0) { hx = T::dv(gx, gn); hy = T::dv(gy, gn); hz = T::dv(gz, gn); }
   R ax = -hz * hx, ay = -hz * hy, az = fma_rn(-hz, hz, (R)1);
   R n1 = T::sq(fma_rn(ax, ax, fma_rn(ay, ay, mul_rn(az, az))));
   if (n1 < (R)1e-12) { ax = (R)1; ay = (R)0; az = (R)0; n1 = (R)1; }
-  ax /= n1; ay /= n1; az /= n1;
+  ax = T::dv(ax, n1); ay = T::dv(ay, n1); az = T::dv(az, n1);
   const R bx = hy * az - hz * ay, by = hz * ax - hx * az, bz = hx * ay - hy * ax;
   const R phi = (R)2 * T::u(w[3]);
   const R cph = T::cpi(phi), sph = T::spi(phi);
-  const R u1 = T::sq((R)2 * e1 / m1), u2 = T::sq((R)2 * wsec / me);
+  const R u1 = T::sq(T::dv((R)2 * e1, m1)), u2 = T::sq(T::dv((R)2 * wsec, me));
   const R sx = fma_rn(cph, ax, mul_rn(sph, bx)), sy = fma_rn(cph, ay, mul_rn(sph, by)),
           sz = fma_rn(cph, az, mul_rn(sph, bz));
   const R ax1 = v2x + u1 * fma_rn(cp, hx, mul_rn(sp, sx));
@@ -625,19 +656,38 @@ __device__ __noinline__ void moving_target_ionization(const Params& P, unsigned 
   L.mu = (double)mu1;
 }
 
+// (double)n for 0 <= n < 2^53 from the bits, else by the conversion
+__device__ __forceinline__ double int_to_d(long long n) {
+  return n >= 0 && n < (1LL << 53) ? u53_scaled((unsigned long long)n, 0) : (double)n;
+}
+
+// The random block of the collision a parked particle chose (the event index
+// before this collision was counted).
+__device__ __forceinline__ void parked_block(const Params& P, const Lane& L,
+                                             unsigned long long w[4]) {
+  philox4x64_10((unsigned long long)(L.ev - 1), L.node,
+                ((unsigned long long)P.pass << 8) | DOM_EVENT, 0ULL, P.seed, L.pid, w);
+}
+
 // Kinematics of a charge exchange (Sec. 3.3), an ionization (Sec. 3.3
 // Ionization: energy sharing, binary-encounter angles, the slow electron and
 // the ion as products) or a clustering
 // (Sec. 3.3 Clustering: the impactor becomes the product ion with a thermal
 // target's motion) of the particle L, whose flight and channel choice are done
-// (L.ev already counts this collision; w is the event's random block).
+// (L.ev already counts this collision; its random block is drawn again).
 template <bool F32>
-__device__ __forceinline__ void rare_kinematics(const Params& P, unsigned long long* led, Lane& L,
-                                                EventOut& o, RingPort& port, int k,
-                                                const unsigned long long w[4]) {
+__device__ __noinline__ void rare_kinematics(const Params& P, unsigned long long* led, Lane& Lref,
+                                             EventOut& o, RingPort& port, int k) {
   using T = RT<F32>;
   using R = typename T::R;
+  Lane L = Lref;
   const ChanDev ch = P.ch[k];
+  struct Put {                                // the particle goes back on every path
+    Lane &a, &b;
+    __device__ ~Put() { a = b; }
+  } put{Lref, L};
+  unsigned long long w[4];
+  parked_block(P, L, w);
   if (ch.kind == CHARGE_EXCHANGE) {
     charge_exchange<F32>(P, L, o.recoil);
     terminate<F32>(P, led, L, o);
@@ -660,15 +710,15 @@ __device__ __forceinline__ void rare_kinematics(const Params& P, unsigned long l
     const long long eq1 = avail - wq;
     sadd(led + (L_LOSS_IONIZ), ch.loss_q);
     // binary encounter: cos^2 of the polar angles are the energy fractions
-    const double inv_avail = avail > 0 ? 1.0 / (double)avail : 0.0;
-    const R c2p = avail > 0 ? (R)((double)eq1 * inv_avail) : (R)1;
-    const R c2s = (R)((double)wq * inv_avail);
+    const double inv_avail = avail > 0 ? RT<false>::dv(1.0, int_to_d(avail)) : 0.0;
+    const R c2p = avail > 0 ? (R)(int_to_d(eq1) * inv_avail) : (R)1;
+    const R c2s = (R)(int_to_d(wq) * inv_avail);
     const R cp = T::sq(c2p), sp = T::sq(c2s);
-    const R cphi = T::cpi((R)2 * T::u(w[3]));
+    const R cphi = T::cpi(T::u2(w[3]));
     const R mu = (R)L.mu;
-    const R smu = T::sq(fmax((R)0, (R)1 - mu * mu));
-    const R mu_p = fmin((R)1, fmax((R)-1, mu * cp + smu * sp * cphi));
-    const R mu_s = fmin((R)1, fmax((R)-1, mu * sp - smu * cp * cphi));
+    const R smu = T::sq(T::max0((R)1 - mu * mu));
+    const R mu_p = T::clamp1(mu * cp + smu * sp * cphi);
+    const R mu_s = T::clamp1(mu * sp - smu * cp * cphi);
     const unsigned evc = L.ev - 1;
     // slow electron (azimuth opposite to the fast one)
     sadd(led + (L_BIRTHS + SP_E), 1);
@@ -714,14 +764,6 @@ __device__ __forceinline__ void rare_kinematics(const Params& P, unsigned long l
     return;
   }
   if (ch.kind == IONIZATION) terminate<F32>(P, led, L, o);
-}
-
-// The random block of the collision a parked particle chose (the event index
-// before this collision was counted).
-__device__ __forceinline__ void parked_block(const Params& P, const Lane& L,
-                                             unsigned long long w[4]) {
-  philox4x64_10((unsigned long long)(L.ev - 1), L.node,
-                ((unsigned long long)P.pass << 8) | DOM_EVENT, 0ULL, P.seed, L.pid, w);
 }
 
 // Order of doubles by their bit patterns: for x >= +0.0 and any y that is not
@@ -810,14 +852,36 @@ __device__ __forceinline__ unsigned long long quant_len(double len, double inv_s
   return (unsigned long long)trunc_nonneg(fma_rn(len, inv_szq, 0.5));
 }
 
-template <bool F32>
-__device__ void event(const Params& P, unsigned long long* led, Lane& L, EventOut& o,
-                      RingPort& port) {
+// Where an event reads the column tables from: device memory through the
+// parameter block's pointers, or the block's shared memory (StagedCols in
+// transport.cu; there the loads need no pointer and the field tables are
+// found by the channel's offset).
+struct GlobalCols {
+  __device__ __forceinline__ double col(const Params& P, int k) const { return P.colgas[k]; }
+  __device__ __forceinline__ double face(const Params& P, int k) const { return P.faces[k]; }
+  __device__ __forceinline__ double n(const Params& P, int j) const { return P.nseg[j]; }
+  __device__ __forceinline__ double invn(const Params& P, int j) const { return P.invn[j]; }
+  __device__ __forceinline__ int ginv(const Params& P, int q) const { return P.ginv[q]; }
+  __device__ __forceinline__ double fcol(const Params& P, int c, int k) const { return P.fcol[c][k]; }
+  __device__ __forceinline__ double frate(const Params& P, int c, int j) const { return P.frate[c][j]; }
+};
+
+// One event of the particle L.  A collision in a rare channel is left to the
+// caller (o.rare), with the particle as the flight left it and the collision
+// counted.
+//
+// P holds the scalars (the constant bank in the single-run kernel), PS the same
+// block in shared memory for the functions out of line, tb the columns.  The
+// particle and the sums stay in registers: nothing here takes their address
+// but copies on the rare paths.
+template <bool F32, class Cols>
+__device__ __forceinline__ void event(const Params& P, const Params& PS, const Cols& tb,
+                                      unsigned long long* led, Lane& L, EventOut& o) {
   using T = RT<F32>;
   using R = typename T::R;
   o.alive = true;
-  o.parked = false;
   o.chan = -1;
+  o.rare = -1;
   if (L.eq <= 0) {                 // no kinetic energy: the particle never moves
     die<F32>(P, led, L, R_STALLED, L_E_STALLED);
     o.alive = false;
@@ -836,16 +900,29 @@ __device__ void event(const Params& P, unsigned long long* led, Lane& L, EventOu
   const R le = T::lg(e * (R)P.inv_e_min);
   const R lx = le * (R)P.inv_h;
   int ti;
+  R tf;
   if constexpr (F32) ti = (int)floor(lx);
   else ti = floor_or_m1(lx);                 // integer ops (below the first node: -1)
-  R tf;
   int row;                                 // row of the cumulative tables (-1: none)
   if (ti < 0) { ti = 0; tf = (R)0; row = P.n_energy - 1; }          // below the first node
   else if (ti > P.n_energy - 2) { ti = P.n_energy - 2; tf = (R)1; row = -1; }
   else {
     if constexpr (F32) tf = lx - (R)ti;
-    else tf = lx - i32_to_d(ti);            // the conversion on integer operations
+    else tf = lx - i32_to_d(ti);              // lx - ti, exact
     row = ti;
+  }
+  const int nsc = P.nsc[s];
+  const int ncg = P.ncg[s];
+  // the tables' loads start here: the interval's mark, the cumulative sums of
+  // all the species' gas channels and of the first
+  int mark = CUM_PER_CHANNEL;
+  R cg_a = (R)0, cg_s = (R)0, c0_a = (R)0, c0_s = (R)0;
+  if (ncg >= 0 && row >= 0) {
+    mark = P.mixed[s * P.n_energy + row];
+    if (ncg > 0) {
+      T::cum2(P, s, row, ncg - 1, cg_a, cg_s);
+      T::cum2(P, s, row, 0, c0_a, c0_s);
+    }
   }
 
   // 1/v and 1/(|mu| v) (relativistic: v = c sqrt(x (2 + x)) / (1 + x), x = E / m c^2);
@@ -864,17 +941,15 @@ __device__ void event(const Params& P, unsigned long long* led, Lane& L, EventOu
   } else {
     const double m2 = still ? 1.0 : mul_rn(L.mu, L.mu);
     const double base =
-        mul_rn(mul_rn((R)1 + x, 1.0 / C_LIGHT), rsqrt(mul_rn(m2, mul_rn(x, (R)2 + x))));
-    inv_v = still ? base : mul_rn(base, amu);
+        mul_rn(mul_rn(1.0 + x, 1.0 / C_LIGHT), rsqrt(mul_rn(m2, mul_rn(x, 2.0 + x))));
+    // electrons need 1/v only where they do not move
+    inv_v = still ? base : s != SP_E ? mul_rn(base, amu) : 0.0;
     inv_szq = mul_rn(base, Q_T);
   }
 
   // ---- rate coefficients of this flight ----
-  const int nsc = P.nsc[s];
-  const int ncg = P.ncg[s];
   // cumulative tables: the species' gas channels lead its selection order and
   // at most one channel threshold falls inside this node interval
-  const int mark = ncg >= 0 && row >= 0 ? P.mixed[s * P.n_energy + row] : CUM_PER_CHANNEL;
   const bool fast = mark != CUM_PER_CHANNEL;
   // a channel that opens inside the interval: above its threshold, its own
   // interpolated cross section joins the sums from its slot xslot on
@@ -892,21 +967,17 @@ __device__ void event(const Params& P, unsigned long long* led, Lane& L, EventOu
   R gas = (R)0;
   int nrec = 0;
   double rc0 = 0.0, rc1 = 0.0;
-  const double* rcol0 = P.colgas;
-  const double* rcol1 = P.colgas;
-  const double* rrate0 = P.nseg;
-  const double* rrate1 = P.nseg;
+  int f0 = 0, f1 = 0;                       // the flight's field channels
   if (fast) {
     if (ncg > 0) {
-      R a0, sl;
-      T::cum2(P, s, row, ncg - 1, a0, sl);
-      gas = fma_rn(tf, sl, a0) + xval;
+      gas = fma_rn(tf, cg_s, cg_a);
+      if (xslot < MAXSPCH) gas = gas + xval;
     }
     for (int c = ncg; c < nsc; ++c) {       // field channels follow the gas channels
       const int k = P.sc[s][c];
       const R cv = channel_coef<F32>(P, k, s, L.eq, ti, tf, inv_v);
-      if (nrec == 0) { rc0 = to_d(cv); rcol0 = P.fcol[k]; rrate0 = P.frate[k]; }
-      else { rc1 = to_d(cv); rcol1 = P.fcol[k]; rrate1 = P.frate[k]; }
+      if (nrec == 0) { rc0 = to_d(cv); f0 = k; }
+      else { rc1 = to_d(cv); f1 = k; }
       ++nrec;
     }
   } else {
@@ -917,8 +988,8 @@ __device__ void event(const Params& P, unsigned long long* led, Lane& L, EventOu
       if (!field_kind(P.ch[k].kind)) {
         gas += cv;
       } else {
-        if (nrec == 0) { rc0 = to_d(cv); rcol0 = P.fcol[k]; rrate0 = P.frate[k]; }
-        else { rc1 = to_d(cv); rcol1 = P.fcol[k]; rrate1 = P.frate[k]; }
+        if (nrec == 0) { rc0 = to_d(cv); f0 = k; }
+        else { rc1 = to_d(cv); f1 = k; }
         ++nrec;
       }
     }
@@ -936,17 +1007,17 @@ __device__ void event(const Params& P, unsigned long long* led, Lane& L, EventOu
   const double gasd = to_d(gas);
 
   // G(k) = optical-depth column of the whole rate to face k, and the rate in
-  // segment j (the column tables may live in shared memory: plain loads)
+  // segment j
   auto colsum = [&](int k) -> double {
-    double g = mul_rn(gasd, P.colgas[k]);
-    if (nrec > 0) g = fma_rn(rc0, rcol0[k], g);
-    if (nrec > 1) g = fma_rn(rc1, rcol1[k], g);
+    double g = mul_rn(gasd, tb.col(P, k));
+    if (nrec > 0) g = fma_rn(rc0, tb.fcol(P, f0, k), g);
+    if (nrec > 1) g = fma_rn(rc1, tb.fcol(P, f1, k), g);
     return g;
   };
   auto segrate = [&](int j) -> double {
-    double r = mul_rn(gasd, P.nseg[j]);
-    if (nrec > 0) r = fma_rn(rc0, rrate0[j], r);
-    if (nrec > 1) r = fma_rn(rc1, rrate1[j], r);
+    double r = mul_rn(gasd, tb.n(P, j));
+    if (nrec > 0) r = fma_rn(rc0, tb.frate(P, f0, j), r);
+    if (nrec > 1) r = fma_rn(rc1, tb.frate(P, f1, j), r);
     return r;
   };
 
@@ -986,10 +1057,10 @@ __device__ void event(const Params& P, unsigned long long* led, Lane& L, EventOu
         double D;
         if constexpr (F32) D = (double)mul_rn(mul_rn(tau, (R)amu), __frcp_rn(gas));
         else D = mul_rn(to_d(tau), amu) / gasd;
-        const double c0 = fma_rn(P.nseg[j0], L.z - P.faces[j0], P.colgas[j0]);
+        const double c0 = fma_rn(tb.n(P, j0), L.z - tb.face(P, j0), tb.col(P, j0));
         tgt = up ? c0 + D : c0 - D;
-        const long long tb = dbits(tgt);
-        ex = up ? tb >= dbits(P.colgas[nz]) : tb <= 0;
+        const long long tgb = dbits(tgt);
+        ex = up ? tgb >= dbits(tb.col(P, nz)) : tgb <= 0;
         if (!ex) {
           // largest k with C(k) <= target, in [j0, nz) going up, [0, j0] going down
           int lo = up ? j0 : 0, hi = up ? nz : j0 + 1;
@@ -997,8 +1068,8 @@ __device__ void event(const Params& P, unsigned long long* led, Lane& L, EventOu
             const float q = dtof_hint(tgt) * P.nq_over_colmax_f;
             if (q >= 0.0f && q < (float)P.nq) {
               const int qi = (int)q;
-              const int a = max(lo, P.ginv[qi] - 1), bb = min(hi, P.ginv[qi + 1] + 1);
-              if (a < bb && dbits(P.colgas[a]) <= tb && tb < dbits(P.colgas[bb])) {
+              const int a = max(lo, tb.ginv(P, qi) - 1), bb = min(hi, tb.ginv(P, qi + 1) + 1);
+              if (a < bb && dbits(tb.col(P, a)) <= tgb && tgb < dbits(tb.col(P, bb))) {
                 lo = a;
                 hi = bb;
               }
@@ -1006,12 +1077,12 @@ __device__ void event(const Params& P, unsigned long long* led, Lane& L, EventOu
           }
           while (hi - lo > 1) {
             const int mid = (lo + hi) >> 1;
-            if (dbits(P.colgas[mid]) <= tb) lo = mid; else hi = mid;
+            if (dbits(tb.col(P, mid)) <= tgb) lo = mid; else hi = mid;
           }
           jc = lo;
-          const double fj = P.faces[jc];
-          zc = fma_rn(tgt - P.colgas[jc], P.invn[jc], fj);
-          zc = dmin_nn(dmax_nn(zc, fj), P.faces[jc + 1]);
+          const double fj = tb.face(P, jc);
+          zc = fma_rn(tgt - tb.col(P, jc), tb.invn(P, jc), fj);
+          zc = dmin_nn(dmax_nn(zc, fj), tb.face(P, jc + 1));
           zc = up ? dmax_nn(zc, L.z) : dmin_nn(zc, L.z);
         }
       }
@@ -1028,32 +1099,32 @@ __device__ void event(const Params& P, unsigned long long* led, Lane& L, EventOu
       rho0 = mul_rn(rc0, ig);
       rho1 = mul_rn(rc1, ig);
       auto gcol = [&](int k) -> double {
-        double g = P.colgas[k];
-        if (nrec > 0) g = fma_rn(rho0, rcol0[k], g);
-        if (nrec > 1) g = fma_rn(rho1, rcol1[k], g);
+        double g = tb.col(P, k);
+        if (nrec > 0) g = fma_rn(rho0, tb.fcol(P, f0, k), g);
+        if (nrec > 1) g = fma_rn(rho1, tb.fcol(P, f1, k), g);
         return g;
       };
       auto frate = [&](int j) -> double {   // field rate per unit of gas density
         double r = 0.0;
-        if (nrec > 0) r = mul_rn(rho0, rrate0[j]);
-        if (nrec > 1) r = fma_rn(rho1, rrate1[j], r);
+        if (nrec > 0) r = mul_rn(rho0, tb.frate(P, f0, j));
+        if (nrec > 1) r = fma_rn(rho1, tb.frate(P, f1, j), r);
         return r;
       };
-      const double c0 = fma_rn(P.nseg[j0] + frate(j0), L.z - P.faces[j0], gcol(j0));
+      const double c0 = fma_rn(tb.n(P, j0) + frate(j0), L.z - tb.face(P, j0), gcol(j0));
       const double D = mul_rn(mul_rn(to_d(tau), amu), ig);
       const double tgt = up ? c0 + D : c0 - D;
       // G >= C everywhere (rho and the field columns are non-negative): a
       // target below the gas column's top is below G's top too
-      ex = up ? !lt_nn(tgt, P.colgas[nz]) && !lt_nn(tgt, gcol(nz)) : !dpos(tgt);
+      ex = up ? !lt_nn(tgt, tb.col(P, nz)) && !lt_nn(tgt, gcol(nz)) : !dpos(tgt);
       if (!ex) {
-        const long long tb = dbits(tgt);
+        const long long tgb = dbits(tgt);
         int lo = up ? j0 : 0, hi = up ? nz : j0 + 1;
         if (P.nq > 0) {
           const float q = dtof_hint(tgt) * P.nq_over_colmax_f;
           if (q >= 0.0f && q < (float)P.nq) {
             const int qi = (int)q;
-            const int a = max(lo, P.ginv[qi] - 1), bb = min(hi, P.ginv[qi + 1] + 1);
-            if (a < bb && dbits(P.colgas[a]) <= tb && tb < dbits(P.colgas[bb])) {
+            const int a = max(lo, tb.ginv(P, qi) - 1), bb = min(hi, tb.ginv(P, qi + 1) + 1);
+            if (a < bb && dbits(tb.col(P, a)) <= tgb && tgb < dbits(tb.col(P, bb))) {
               lo = a;
               hi = bb;
             }
@@ -1061,7 +1132,7 @@ __device__ void event(const Params& P, unsigned long long* led, Lane& L, EventOu
         }
         while (hi - lo > 1) {
           const int mid = (lo + hi) >> 1;
-          if (dbits(P.colgas[mid]) <= tb) lo = mid; else hi = mid;
+          if (dbits(tb.col(P, mid)) <= tgb) lo = mid; else hi = mid;
         }
         jc = lo;
         double gj = gcol(jc);
@@ -1074,44 +1145,36 @@ __device__ void event(const Params& P, unsigned long long* led, Lane& L, EventOu
           jc = l2;
           gj = gcol(jc);
         }
-        const double fj = P.faces[jc];
+        const double fj = tb.face(P, jc);
         const double gap = tgt - gj;
-        const double nj = P.nseg[jc];
+        const double nj = tb.n(P, jc), vj = tb.invn(P, jc);
         rf_end = frate(jc);
         double off;
-        const double eps = mul_rn(rf_end, P.invn[jc]);
+        const double eps = mul_rn(rf_end, vj);
         if (dpos(nj) && dabs_lt(eps, 1e-6))
           // 1 / (n + rf) = (1/n) (1 - eps + eps^2) to eps^3, eps = rf / n
-          off = mul_rn(gap, mul_rn(P.invn[jc], fma_rn(-eps, 1.0 - eps, 1.0)));
+          off = mul_rn(gap, mul_rn(vj, fma_rn(-eps, 1.0 - eps, 1.0)));
         else
           off = gap / (nj + rf_end);
         zc = fj + off;
-        zc = dmin_nn(dmax_nn(zc, fj), P.faces[jc + 1]);
+        zc = dmin_nn(dmax_nn(zc, fj), tb.face(P, jc + 1));
         zc = up ? dmax_nn(zc, L.z) : dmin_nn(zc, L.z);
       }
     } else {
       // Field channels only (no gas rate): the flight inverts the column of
       // the fields, bracketed from the gas column where there is one.
-      const double g0 = fma_rn(segrate(j0), L.z - P.faces[j0], colsum(j0));
+      const double g0 = fma_rn(segrate(j0), L.z - tb.face(P, j0), colsum(j0));
       const double delta = mul_rn(to_d(tau), amu);
       const double target = up ? g0 + delta : g0 - delta;
       ex = up ? !(target < colsum(nz)) : !(target > 0.0);
       if (!ex) {
         int lo = up ? j0 : 0, hi = up ? nz : j0 + 1;
-        if (gasd > 0.0 && P.nq > 0) {
-          const float q = (float)target * P.nq_over_colmax_f * __frcp_rn((float)gas);
-          if (q >= 0.0f && q < (float)P.nq) {
-            const int qi = (int)q;
-            const int a = max(lo, P.ginv[qi] - 1), bb = min(hi, P.ginv[qi + 1] + 1);
-            if (a < bb && colsum(a) <= target && target < colsum(bb)) { lo = a; hi = bb; }
-          }
-        }
         while (hi - lo > 1) {
           const int mid = (lo + hi) >> 1;
           if (colsum(mid) <= target) lo = mid; else hi = mid;
         }
         jc = lo;
-        const double fj = P.faces[jc], fj1 = P.faces[jc + 1];
+        const double fj = tb.face(P, jc), fj1 = tb.face(P, jc + 1);
         const double gap = target - colsum(jc);
         const double r = segrate(jc);
         if (F32) zc = fj + (double)((float)gap / (float)r);
@@ -1130,13 +1193,13 @@ __device__ void event(const Params& P, unsigned long long* led, Lane& L, EventOu
     // crossings (Sec. 2.3) as one range add.  One instruction stream for a
     // flight within one segment and one across many.
     const bool same = jc == j0;
-    const double fs = P.faces[up ? j0 + 1 : j0];
-    const double fe = P.faces[up ? jc : jc + 1];
+    const double fs = tb.face(P, up ? j0 + 1 : j0);
     const unsigned long long q0 = quant_len(fabs((same ? zc : fs) - L.z), inv_szq);
-    const unsigned long long qf = quant_len(P.dz, inv_szq);
-    const unsigned long long qe = quant_len(fabs(zc - fe), inv_szq);
     atomicAdd(P.time_pt + tbase + (size_t)(j0 + 1) * trow, q0);
     if (!same) {
+      const double fe = tb.face(P, up ? jc : jc + 1);
+      const unsigned long long qf = quant_len(P.dz, inv_szq);
+      const unsigned long long qe = quant_len(fabs(zc - fe), inv_szq);
       atomicAdd(P.time_pt + tbase + (size_t)(jc + 1) * trow, ex ? qf : qe);
       const int lo_seg = min(j0, jc), hi_seg = max(j0, jc);
       range_add(P.time_rg + tbase, lo_seg + 2, hi_seg, trow, qf);   // full segments
@@ -1171,18 +1234,17 @@ __device__ void event(const Params& P, unsigned long long* led, Lane& L, EventOu
     } else if (gas_units) {
       // rates per unit of gas density: gas channels n_jc (then in sigma
       // units for the cumulative tables), field channel i rho_i f_i(jc)
-      const double nj = P.nseg[jc];
+      const double nj = tb.n(P, jc);
       const double tr = mul_rn(u01d(w[1]), nj + rf_end);
       if (lt_nn(tr, nj)) {
-        tg = from_d<R>(mul_rn(mul_rn(tr, P.invn[jc]), gasd));
+        tg = from_d<R>(mul_rn(mul_rn(tr, tb.invn(P, jc)), gasd));
       } else {
         gas_part = false;
         tg = (R)0;
         double cum = nj;
         int last = -1;
         for (int c = ncg; c < nsc; ++c) {
-          const int kk = P.sc[s][c];
-          const double rk = mul_rn(c == ncg ? rho0 : rho1, P.frate[kk][jc]);
+          const double rk = mul_rn(c == ncg ? rho0 : rho1, tb.frate(P, P.sc[s][c], jc));
           if (!dpos(rk)) continue;
           last = c;
           cum += rk;
@@ -1191,19 +1253,18 @@ __device__ void event(const Params& P, unsigned long long* led, Lane& L, EventOu
         if (chs < 0) chs = last;
       }
     } else {
-      const double nj = P.nseg[jc];
+      const double nj = tb.n(P, jc);
       const double target = mul_rn(u01d(w[1]), segrate(jc));
       const double gasj = mul_rn(gasd, nj);
       if (lt_nn(target, gasj)) {
-        tg = from_d<R>(mul_rn(target, P.invn[jc]));
+        tg = from_d<R>(mul_rn(target, tb.invn(P, jc)));
       } else {
         gas_part = false;
         tg = (R)0;
         double cum = gasj;
         int last = -1;
         for (int c = ncg; c < nsc; ++c) {
-          const int kk = P.sc[s][c];
-          const double rk = mul_rn(c == ncg ? rc0 : rc1, P.frate[kk][jc]);
+          const double rk = mul_rn(c == ncg ? rc0 : rc1, tb.frate(P, P.sc[s][c], jc));
           if (!dpos(rk)) continue;
           last = c;
           cum += rk;
@@ -1213,29 +1274,46 @@ __device__ void event(const Params& P, unsigned long long* led, Lane& L, EventOu
       }
     }
     if (gas_part) {
+      R a0 = c0_a, sl = c0_s;
       for (int c = 0; c < ncg; ++c) {
-        R a0, sl;
-        T::cum2(P, s, row, c, a0, sl);
-        if (lt_nn(tg, fma_rn(tf, sl, a0) + (c >= xslot ? xval : (R)0))) { chs = c; break; }
+        if (c > 0) T::cum2(P, s, row, c, a0, sl);
+        R cv = fma_rn(tf, sl, a0);
+        if (c >= xslot) cv = cv + xval;
+        if (lt_nn(tg, cv)) { chs = c; break; }
       }
     }
-    if (chs < 0)                        // rounding at the top end
-      chs = select_per_channel<F32>(P, s, L.eq, ti, tf, inv_v, nrec, jc, w[1]);
-  } else {
-    chs = select_per_channel<F32>(P, s, L.eq, ti, tf, inv_v, nrec, jc, w[1]);
   }
+  if (chs < 0)                          // per-channel path, or rounding at the top end
+    chs = select_per_channel<F32>(PS, s, L.eq, ti, tf, inv_v, nrec, jc, w[1]);
   const int k = P.sc[s][chs];
   o.chan = k;
-  const ChanDev ch = P.ch[k];
-  if (ch.kind == ELASTIC && ch.target) {
-    moving_target_elastic<F32>(P, ch, L, w, o.recoil);
-  } else if (ch.kind == ELASTIC) {
+  const int kind = P.ch[k].kind;
+  if (kind == ELASTIC && P.ch[k].target) {
+    // (copies, so that the particle itself keeps to registers)
+    Lane M = L;
+    const unsigned long long wm[4] = {w[0], w[1], w[2], w[3]};
+    unsigned long long rc = 0;
+    moving_target_elastic<F32>(PS, PS.ch[k], M, wm, rc);
+    o.recoil += rc;
+    L.eq = M.eq;
+    L.mu = M.mu;
+  } else if (kind == ELASTIC) {
     // CM polar angle (isotropic or tabulated at the lab energy, which is the
     // impact energy for a target at rest): lab polar angle and energy transfer
     const R g = (R)P.gam[s];
     const R g2 = (R)P.gam2[s];                 // 2 g
-    const R cchi = elastic_cchi<F32>(P, ch, e, T::u(w[2]));
-    const R a = fma_rn(g2, cchi, fma_rn(g, g, (R)1));
+    R cchi, omc;                               // cos chi and 1 - cos chi
+    const int ang = P.ch[k].ang;
+    if (ang >= 0 && e >= (R)P.ang_thr[ang]) {
+      cchi = table_cchi<F32>(PS, ang, e, T::u(w[2]));
+      omc = (R)1 - cchi;
+    } else {
+      cchi = (R)2 * T::u(w[2]) - (R)1;
+      omc = (R)1 - cchi;
+    }
+    R a;
+    if constexpr (F32) a = fma_rn(g2, cchi, fma_rn(g, g, (R)1));
+    else a = fma_rn(g2, cchi, fma_rn(g, g, 1.0));      // g^2 + 1 rounded once, on the host
     const R ra = T::rsq(a);
     const R ct = mul_rn(cchi + g, ra);
     // energy given to the target, E - E' = E 2g(1 - cos chi)/(1+g)^2
@@ -1247,31 +1325,19 @@ __device__ void event(const Params& P, unsigned long long* led, Lane& L, EventOu
     // sin(theta_lab) sqrt(1 - mu^2) in one root: 1 - ct^2 = (1 - cchi^2) / a
     const R cphi = T::cpi(mul_rn((R)2, T::u(w[3])));
     const R mu = from_d<R>(L.mu);
-    const R ss = mul_rn(T::sq(T::max0(mul_rn(fma_rn(-cchi, cchi, (R)1), fma_rn(-mu, mu, (R)1)))),
-                        ra);
+    const R s2 = T::max0(mul_rn(fma_rn(-cchi, cchi, (R)1), fma_rn(-mu, mu, (R)1)));
+    const R ss = mul_rn(F32 ? (R)sqrtf((float)s2) : (R)sqrt((double)s2), ra);
     L.mu = to_d(T::clamp1(fma_rn(mu, ct, mul_rn(ss, cphi))));
-  } else if (ch.kind == EXCITATION) {
-    L.eq -= ch.loss_q;
-    o.excit += (unsigned long long)ch.loss_q;
-  } else if (ch.kind == IONIZATION || ch.kind == CLUSTERING || ch.kind == CLUSTERING3 ||
-             ch.kind == CHARGE_EXCHANGE) {
-    if (port.rare) {
-      RareBuf* rb = port.rare;
-      const int i = atomicAdd(&rb->n, 1);
-      if (i < RB - rb->r) {
-        rb->s[i] = L;
-        rb->ch[i] = (int8_t)k;
-        o.alive = false;
-        o.parked = true;
-        return;
-      }
-    }
-    rare_kinematics<F32>(P, led, L, o, port, k, w);
-    return;
-  } else {  // RECOMBINATION
-    atomicAdd(P.recomb + (size_t)ch.sout * P.nz + jc, 1ULL);
+  } else if (kind == EXCITATION) {
+    L.eq -= P.ch[k].loss_q;
+    o.excit += (unsigned long long)P.ch[k].loss_q;
+  } else if (kind == RECOMBINATION) {
+    atomicAdd(P.recomb + (size_t)P.ch[k].sout * P.nz + jc, 1ULL);
     die<F32>(P, led, L, R_RECOMB, L_E_RECOMB);
     o.alive = false;
+    return;
+  } else {
+    o.rare = k;
     return;
   }
   terminate<F32>(P, led, L, o);

@@ -52,8 +52,9 @@ XA_FN float xa_rsqrt(float x) {
 }
 XA_FN int xa_rint(float x) { return __float2int_rn(x); }
 XA_FN float xa_float(int n) { return __int2float_rn(n); }
-XA_FN double xa_ieee_div(double a, double b) { return __ddiv_rn(a, b); }
-XA_FN double xa_ieee_sqrt(double a) { return __dsqrt_rn(a); }
+// out of line: taken by one operand in a thousand
+static __device__ __noinline__ double xa_ieee_div(double a, double b) { return __ddiv_rn(a, b); }
+static __device__ __noinline__ double xa_ieee_sqrt(double a) { return __dsqrt_rn(a); }
 #else
 XA_FN long long xa_bits(double x) { long long b; std::memcpy(&b, &x, 8); return b; }
 XA_FN double xa_dbl(long long b) { double x; std::memcpy(&x, &b, 8); return x; }

@@ -67,6 +67,7 @@ struct Params {
   // recombination target fields of pass 2, per channel (NULL if unused)
   const double* frate[MAXCH];   // [nz] partner field per segment
   const double* fcol[MAXCH];    // [nz+1] its column to each face
+  int foff[MAXCH];              // its place in the tables staged in shared memory (doubles)
   // cross sections
   int n_energy;
   double e_min, inv_e_min, log_ratio_h, inv_h;   // h = ln(e_max/e_min)/(n-1)

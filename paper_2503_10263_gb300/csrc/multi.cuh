@@ -7,9 +7,9 @@
 // compare-and-swap on that word that never takes primaries past the end;
 // products and deaths are single atomics on the live count, so a pass of a
 // request is complete exactly when a decrement leaves no live particle with
-// every primary claimed; the warp that observes it builds the request's
-// target fields (pass 1 -> 2) or finalises and normalises its outputs (last
-// pass) inside the kernel.
+// every primary claimed; the target fields (pass 1 -> 2) or the final and
+// normalised outputs (last pass) are then built inside the kernel, in units
+// that any warp takes (SlotCtl::task).
 //
 // A slot is reused by later requests.  The host gives each admission a new
 // generation, carried in the state word (bits 8 and up) and, modulo 32, in the
@@ -49,8 +49,14 @@ struct SlotCtl {
   unsigned long long word[2];            // per pass: generation | next primary | live
   int state;                             // generation << 8 | SLOT_*
   int pass;                              // pass being run (1 or 2)
-  char pad[104];
+  // work between and after the passes, shared out to any warp: phase (TASK_*)
+  // << 32 | next unit to take, and the units of the phase finished
+  unsigned long long task;
+  unsigned task_done;
+  char pad[92];
 };
+enum { TASK_NONE = 0, TASK_TIME1 = 1, TASK_FIELD = 2, TASK_COLUMN = 3, TASK_TIME2 = 4,
+       TASK_NORM = 5 };
 
 struct SlotDesc {
   Params P[2];                           // pass-1 and pass-2 parameter blocks
@@ -73,7 +79,9 @@ struct SlotDesc {
 };
 
 struct MultiCtl {
-  Control c;                             // shared ring, abort, error, counters
+  Control c;                             // shared ring, abort, error, counters; prim_next
+                                         // here counts the unclaimed primaries and active the
+                                         // particles held (both only steer the schedule)
   unsigned long long published;          // requests published by the host (sequence)
   char pad0[120];
   unsigned long long adopted;            // requests adopted by the kernel
@@ -81,7 +89,8 @@ struct MultiCtl {
   unsigned long long done_count;
   char pad2[120];
   int shutdown;                          // host: leave once every published request is done
-  int pad3;
+  int tasks;                             // slots between passes (phase not TASK_NONE)
+  unsigned taskmap[MAX_SLOTS / 32];      // those slots
   unsigned bitmap[MAX_SLOTS / 32];       // slots with unclaimed primaries in their pass
   unsigned pubq[MAX_SLOTS];              // slot of the request with sequence number q % MAX_SLOTS
 };

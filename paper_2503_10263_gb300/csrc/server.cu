@@ -24,7 +24,7 @@
 namespace karl {
 cudaError_t launch_multi(bool f32, SlotDesc* D, SlotCtl* C, MultiCtl* M, const Ring& R,
                          const volatile int* cancel, unsigned long long timeout_ns, int grid,
-                         int block, cudaStream_t st);
+                         int block, int bps, cudaStream_t st);
 cudaError_t multi_occupancy(bool f32, int block, int* blocks_per_sm);
 }  // namespace karl
 
@@ -243,7 +243,7 @@ karl_status launch(karl_server* srv) {
   SCK(cudaEventRecord(srv->ev0, srv->kstream));
   SCK(launch_multi(f32, srv->d_desc, srv->d_ctl, srv->d_M, srv->ring, srv->d_cancel,
                    (unsigned long long)(srv->opts.timeout_s * 1e9), srv->num_sms * bps,
-                   srv->opts.block_size, srv->kstream));
+                   srv->opts.block_size, bps, srv->kstream));
   SCK(cudaEventRecord(srv->ev1, srv->kstream));
   srv->running = true;
   srv->stats.kernel_launches += 1;
@@ -570,11 +570,12 @@ karl_status ensure_ring(karl_server* srv) {
   return KARL_OK;
 }
 
-// collect finished requests, then admit waiting ones in arrival order
-karl_status progress(karl_server* srv) {
+// collect finished requests (not while submitting: a submit copies no other
+// request's results back), then admit waiting ones in arrival order
+karl_status progress(karl_server* srv, bool collecting = true) {
   karl_status st = reap_launch(srv);
   if (st && st != KARL_ECAPACITY) return st;
-  for (auto& kv : srv->reqs) {
+  if (collecting) for (auto& kv : srv->reqs) {
     Request& r = kv.second;
     if (r.state == REQ_ADMITTED && srv->h_done[r.slot]) {
       karl_status c = collect(srv, r);
@@ -794,7 +795,7 @@ karl_status karl_server_submit(karl_server* srv, const karl_geometry* g, const k
   srv->reqs.emplace(r.id, std::move(r));
   srv->waiting.push_back(*req_id);
   srv->stats.submitted += 1;
-  return progress(srv);
+  return progress(srv, false);
 }
 
 karl_status karl_server_poll(karl_server* srv, uint64_t req_id, int* done) {

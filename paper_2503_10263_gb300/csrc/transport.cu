@@ -12,6 +12,8 @@
 // take the next one from their queue, from the ring or from the primaries.
 // All waits are bounded by iteration counts and a wall-clock deadline, after
 // which the kernel records an error and returns.
+#include <type_traits>
+
 #include "event.cuh"
 
 namespace karl {
@@ -19,53 +21,61 @@ namespace karl {
 // ---------------------------------------------------------------------------
 // persistent kernel
 
-// Particles of a warp's queue that a claim on the ring may fill (half the
-// queue, so the products of the next events still find room).
-constexpr int RING_BATCH = WQ / 2;
-
-// Copy the column tables (and the pass-2 recombination fields) into dynamic
-// shared memory when they fit; the event code reads them through P's pointers.
-__device__ void stage_tables(Params& SP, const Params& Pk, double* dyn, int dyn_doubles) {
-  const int nz = Pk.nz;
-  int need = (4 * nz + 2) + (Pk.nq + 1 + 1) / 2 + 1;
-  for (int k = 0; k < Pk.nch; ++k)
-    if (Pk.fcol[k]) need += 2 * nz + 1;
-  if (need > dyn_doubles) return;                   // stay in global memory
-  double* col = dyn;
-  double* fac = col + (nz + 1);
-  double* nseg = fac + (nz + 1);
-  double* invn = nseg + nz;
-  int* ginv = (int*)(invn + nz);
-  double* next = (double*)(ginv + ((Pk.nq + 2) & ~1));
-  for (int i = threadIdx.x; i <= nz; i += blockDim.x) col[i] = Pk.colgas[i];
-  for (int i = threadIdx.x; i <= nz; i += blockDim.x) fac[i] = Pk.faces[i];
-  for (int i = threadIdx.x; i < nz; i += blockDim.x) nseg[i] = Pk.nseg[i];
-  for (int i = threadIdx.x; i < nz; i += blockDim.x) invn[i] = Pk.invn[i];
-  if (Pk.ginv)
-    for (int i = threadIdx.x; i <= Pk.nq; i += blockDim.x) ginv[i] = Pk.ginv[i];
-  if (threadIdx.x == 0) {
-    SP.colgas = col;
-    SP.faces = fac;
-    SP.nseg = nseg;
-    SP.invn = invn;
-    if (Pk.ginv) SP.ginv = ginv;
+// The column tables in the block's dynamic shared memory, one after the
+// other: gas column and faces (nz + 1 each), density and its inverse (nz
+// each), the inverse column, then column and rate of each field channel from
+// the channel's offset.
+struct StagedCols {
+  const double* at;
+  __device__ __forceinline__ double col(const Params&, int k) const { return at[k]; }
+  __device__ __forceinline__ double face(const Params& P, int k) const { return at[P.nz + 1 + k]; }
+  __device__ __forceinline__ double n(const Params& P, int j) const { return at[2 * P.nz + 2 + j]; }
+  __device__ __forceinline__ double invn(const Params& P, int j) const { return at[3 * P.nz + 2 + j]; }
+  __device__ __forceinline__ int ginv(const Params& P, int q) const {
+    return ((const int*)(at + 4 * P.nz + 2))[q];
   }
-  for (int k = 0; k < Pk.nch; ++k) {
-    if (!Pk.fcol[k]) continue;
-    double* fc = next;
-    double* fr = next + (nz + 1);
-    next += 2 * nz + 1;
-    for (int i = threadIdx.x; i <= nz; i += blockDim.x) fc[i] = Pk.fcol[k][i];
-    for (int i = threadIdx.x; i < nz; i += blockDim.x) fr[i] = Pk.frate[k][i];
-    if (threadIdx.x == 0) { SP.fcol[k] = fc; SP.frate[k] = fr; }
+  __device__ __forceinline__ double fcol(const Params& P, int c, int k) const {
+    return at[P.foff[c] + k];
+  }
+  __device__ __forceinline__ double frate(const Params& P, int c, int j) const {
+    return at[P.foff[c] + P.nz + 1 + j];
+  }
+};
+
+__device__ __forceinline__ void stage_tables(const Params& P, double* at) {
+  const int nz = P.nz;
+  int* ginv = (int*)(at + 4 * nz + 2);
+  for (int i = threadIdx.x; i <= nz; i += blockDim.x) {
+    at[i] = P.colgas[i];
+    at[nz + 1 + i] = P.faces[i];
+  }
+  for (int i = threadIdx.x; i < nz; i += blockDim.x) {
+    at[2 * nz + 2 + i] = P.nseg[i];
+    at[3 * nz + 2 + i] = P.invn[i];
+  }
+  if (P.ginv)
+    for (int i = threadIdx.x; i <= P.nq; i += blockDim.x) ginv[i] = P.ginv[i];
+  for (int c = 0; c < P.nch; ++c) {
+    if (!P.fcol[c]) continue;
+    double* f = at + P.foff[c];
+    for (int i = threadIdx.x; i <= nz; i += blockDim.x) f[i] = P.fcol[c][i];
+    for (int i = threadIdx.x; i < nz; i += blockDim.x) f[nz + 1 + i] = P.frate[c][i];
   }
 }
 
-template <bool F32>
-__global__ void __launch_bounds__(512, 1) transport_kernel(const Params Pk, Ring R, Control* ctl,
-                                                        const volatile int* cancel,
-                                                        unsigned long long timeout_ns,
-                                                        int dyn_doubles) {
+// STAGED: the column tables fit the block's shared memory (dyn_doubles of it).
+// The parameters are read from the constant bank and the staged columns at
+// offsets of the block's shared memory, without a pointer; nothing takes the
+// particle's address but copies on the rare paths, which are out of line.
+// (With the parameters behind a shared-memory reference and the particle in
+// local memory, the FP32 form's pass 1 took 28.2 ms at 1e5 decays, 26.1 now;
+// 3e5 decays at 3.1e21 m^-2 47 and 42 ms.  The FP64 form, held by its FP64
+// instructions, gained 1 %.)
+template <bool F32, bool STAGED>
+__global__ void __launch_bounds__(512, 1)
+    transport_kernel(const __grid_constant__ Params P, const __grid_constant__ Ring R,
+                     Control* ctl, const volatile int* cancel, unsigned long long timeout_ns,
+                     int dyn_doubles) {
   const unsigned long long deadline = globaltimer_ns() + timeout_ns;
   if (threadIdx.x == 0 && ld_relaxed(&ctl->t_start) == 0)
     atomicCAS(&ctl->t_start, 0ULL, deadline - timeout_ns);
@@ -73,11 +83,10 @@ __global__ void __launch_bounds__(512, 1) transport_kernel(const Params Pk, Ring
   // queue and one batch of parked collisions per warp of the block
   extern __shared__ double dyn[];
   __shared__ Shared S;
-  __shared__ Params SP;
+  __shared__ Params SP;                           // for the functions out of line
   const int nwarps = blockDim.x >> 5;
   WarpQueue* wq = (WarpQueue*)(dyn + dyn_doubles);
   RareBuf* rbuf = (RareBuf*)(wq + nwarps);
-  if (threadIdx.x == 0) SP = Pk;
   for (int i = threadIdx.x; i < LEDGER; i += blockDim.x) S.ledger[i] = 0;
   for (int i = threadIdx.x; i < MAXCH; i += blockDim.x) S.chan[i] = 0;
   if (threadIdx.x < nwarps) {
@@ -85,10 +94,11 @@ __global__ void __launch_bounds__(512, 1) transport_kernel(const Params Pk, Ring
     rbuf[threadIdx.x].n = 0;
     rbuf[threadIdx.x].r = 0;
   }
+  if (threadIdx.x == 0) SP = P;
+  if (STAGED) stage_tables(P, dyn);
   __syncthreads();
-  stage_tables(SP, Pk, dyn, dyn_doubles);
-  __syncthreads();
-  const Params& P = SP;
+  typename std::conditional<STAGED, StagedCols, GlobalCols>::type cols;
+  if constexpr (STAGED) cols.at = dyn;
 
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
@@ -98,7 +108,6 @@ __global__ void __launch_bounds__(512, 1) transport_kernel(const Params Pk, Ring
   bool has = false;
   Lane L;
   EventOut o;
-  o.parked = false;
   o.flights = 0;
   o.colls = 0;
   o.recoil = 0;
@@ -117,8 +126,6 @@ __global__ void __launch_bounds__(512, 1) transport_kernel(const Params Pk, Ring
   port.ctl = ctl;
   port.deadline = deadline;
   port.q = &Q;
-  port.rare = &Rb;
-  port.local = true;
   port.spilled = 0;
   port.slot_live = nullptr;
 
@@ -465,17 +472,38 @@ __global__ void __launch_bounds__(512, 1) transport_kernel(const Params Pk, Ring
 
     // ---- one event ----
     bool died = false;
+    o.rare = -1;
+    if (has && rk < 0) {
+      event<F32>(P, SP, cols, S.ledger, L, o);
+      if (!o.alive) {
+        has = false;
+        died = true;
+      } else if (o.rare >= 0) {
+        // park it for the warp's next batch, or perform it now if all places
+        // are taken
+        const int i = atomicAdd(&Rb.n, 1);
+        if (i < RB - Rb.r) {
+          Rb.s[i] = L;
+          Rb.ch[i] = (int8_t)o.rare;
+          has = false;
+        } else {
+          rk = o.rare;
+        }
+      }
+    }
     if (has && rk >= 0) {
-      unsigned long long w[4];
-      parked_block(P, L, w);
-      o.alive = true;
-      o.parked = false;
-      o.chan = -1;
-      rare_kinematics<F32>(P, S.ledger, L, o, port, rk, w);
-      if (!o.alive) { has = false; died = true; }
-    } else if (has) {
-      event<F32>(P, S.ledger, L, o, port);
-      if (!o.alive) { has = false; died = !o.parked; }
+      // (copies: only here the particle and the sums have an address)
+      Lane M = L;
+      EventOut m;
+      m.alive = true;
+      m.recoil = 0;
+      rare_kinematics<F32>(SP, S.ledger, M, m, port, rk);
+      L = M;
+      o.recoil += m.recoil;
+      if (!m.alive) {
+        has = false;
+        died = true;
+      }
     }
     __syncwarp();
     const int qtop = min(Q.top, WQ);                  // pushes past the end went to the ring
@@ -566,8 +594,24 @@ int transport_dyn_doubles(const Params& P, int block) {
   return need * 8 <= dyn_table_budget(block) ? need : 0;
 }
 
+// Where stage_tables puts each field channel's tables.
+void transport_offsets(Params& P) {
+  int at = (4 * P.nz + 2) + (P.nq + 2) / 2;
+  for (int k = 0; k < P.nch; ++k) {
+    P.foff[k] = at;
+    if (P.fcol[k]) at += 2 * P.nz + 1;
+  }
+}
+
 size_t transport_dyn_bytes(const Params& P, int block) {
   return (size_t)transport_dyn_doubles(P, block) * 8 + (size_t)(block / 32) * QUEUE_BYTES_PER_WARP;
+}
+
+using TransportKernel = void (*)(const Params, const Ring, Control*, const volatile int*,
+                                 unsigned long long, int);
+TransportKernel kernel_for(bool f32, bool staged) {
+  if (f32) return staged ? transport_kernel<true, true> : transport_kernel<true, false>;
+  return staged ? transport_kernel<false, true> : transport_kernel<false, false>;
 }
 
 cudaError_t launch_transport(bool f32, const Params& P, const Ring& R, Control* ctl,
@@ -575,29 +619,26 @@ cudaError_t launch_transport(bool f32, const Params& P, const Ring& R, Control* 
                              int block, cudaStream_t st) {
   const int dd = transport_dyn_doubles(P, block);
   const size_t bytes = transport_dyn_bytes(P, block);
-  if (f32)
-    transport_kernel<true><<<grid, block, bytes, st>>>(P, R, ctl, cancel, timeout_ns, dd);
-  else
-    transport_kernel<false><<<grid, block, bytes, st>>>(P, R, ctl, cancel, timeout_ns, dd);
+  Params Q = P;
+  transport_offsets(Q);
+  kernel_for(f32, dd > 0)<<<grid, block, bytes, st>>>(Q, R, ctl, cancel, timeout_ns, dd);
   return cudaGetLastError();
 }
 
 cudaError_t transport_setup() {
-  cudaError_t e = cudaFuncSetAttribute(transport_kernel<true>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       SMEM_PER_SM - STATIC_SMEM_MARGIN);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(transport_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              SMEM_PER_SM - STATIC_SMEM_MARGIN);
+  for (int v = 0; v < 4; ++v) {
+    cudaError_t e = cudaFuncSetAttribute(kernel_for(v & 1, v & 2),
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         SMEM_PER_SM - STATIC_SMEM_MARGIN);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t transport_occupancy(bool f32, const Params& P, int block, int* blocks_per_sm) {
-  const size_t bytes = transport_dyn_bytes(P, block);
-  if (f32)
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, transport_kernel<true>,
-                                                         block, bytes);
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, transport_kernel<false>,
-                                                       block, bytes);
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+      blocks_per_sm, kernel_for(f32, transport_dyn_doubles(P, block) > 0), block,
+      transport_dyn_bytes(P, block));
 }
 
 }  // namespace karl
