@@ -19,6 +19,7 @@
 #include <vector>
 
 #include "../../include/karl.h"
+#include "exact_arith.cuh"
 #include "host_common.h"
 #include "orbit.cuh"
 
@@ -277,28 +278,68 @@ __global__ void k_check_primaries(const double* z, const double* e, const double
   }
 }
 
-// time = point adds + prefix of range adds, per (species, energy bin)
-__global__ void k_finalize_time(const unsigned long long* pt, const unsigned long long* rg,
-                                unsigned long long* out, int nz, int ntb) {
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= NSP * ntb) return;
-  int s = t / ntb, b = t % ntb;
-  unsigned long long acc = 0;
-  for (int row = 0; row < nz + 2; ++row) {
-    size_t i = ((size_t)s * (nz + 2) + row) * ntb + b;
-    acc += rg[i];
-    out[i] = pt[i] + acc;
-  }
-}
+// The sums along z after a pass, in one launch of FIN_WARPS-warp blocks.  A
+// sum over 1000 rows is a chain of loads when one thread walks it (0.5 ms for
+// the time tally, 0.16 ms for each crossing tally); here the warps of a block
+// each add up a stretch of rows, the stretches' sums are added up over the
+// warps in shared memory, and each warp then writes its stretch.  The sums are
+// integers, so the order does not matter.  At 1000 rows and 64 energy bins
+// 0.83 ms in three launches before, 0.02 ms in one now.
+// Blocks below n_time: time = point adds + prefix of range adds for 32 of the
+// (species, energy bin) columns; the others: face crossings of one species,
+// first +z, then -z (pt NULL).
+constexpr int FIN_WARPS = 32;
 
-__global__ void k_finalize_cross(const unsigned long long* rg, unsigned long long* out, int nz) {
-  int s = threadIdx.x;
-  if (s >= NSP) return;
-  unsigned long long acc = 0;
-  for (int k = 0; k <= nz; ++k) {
-    acc += rg[(size_t)s * (nz + 2) + k];
-    out[(size_t)s * (nz + 1) + k] = acc;
+__global__ void __launch_bounds__(32 * FIN_WARPS)
+    k_finalize(const unsigned long long* pt, const unsigned long long* rg,
+               unsigned long long* out, const unsigned long long* xpos,
+               const unsigned long long* xneg, unsigned long long* cpos, unsigned long long* cneg,
+               int nz, int ntb, int n_time) {
+  __shared__ unsigned long long part[FIN_WARPS][33];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if ((int)blockIdx.x < n_time) {
+    // lane = column, warp = stretch of rows
+    const int col = 32 * blockIdx.x + lane;
+    const bool on = col < NSP * ntb;
+    const int s = on ? col / ntb : 0, b = on ? col % ntb : 0;
+    const size_t at = (size_t)s * (nz + 2) * ntb + b;
+    const int rows = nz + 2, len = (rows + FIN_WARPS - 1) / FIN_WARPS;
+    const int r0 = min(rows, w * len), r1 = min(rows, r0 + len);
+    unsigned long long sum = 0;
+    if (on)
+#pragma unroll 8
+      for (int r = r0; r < r1; ++r) sum += rg[at + (size_t)r * ntb];
+    part[w][lane] = sum;
+    __syncthreads();
+    unsigned long long acc = 0;
+    for (int i = 0; i < w; ++i) acc += part[i][lane];
+    if (on)
+#pragma unroll 8
+      for (int r = r0; r < r1; ++r) {
+        const size_t i = at + (size_t)r * ntb;
+        acc += rg[i];
+        out[i] = pt[i] + acc;
+      }
+    return;
   }
+  // crossings: a stretch of faces per thread
+  const int c = blockIdx.x - n_time, s = c % NSP;
+  const unsigned long long* src = (c < NSP ? xpos : xneg) + (size_t)s * (nz + 2);
+  unsigned long long* dst = (c < NSP ? cpos : cneg) + (size_t)s * (nz + 1);
+  const int n = nz + 1, len = (n + 32 * FIN_WARPS - 1) / (32 * FIN_WARPS);
+  const int k0 = min(n, (int)threadIdx.x * len), k1 = min(n, k0 + len);
+  unsigned long long sum = 0;
+  for (int k = k0; k < k1; ++k) sum += src[k];
+  unsigned long long pre = sum;                      // inclusive over the warp
+  for (int d = 1; d < 32; d <<= 1) {
+    const unsigned long long v = __shfl_up_sync(0xffffffffu, pre, d);
+    if (lane >= d) pre += v;
+  }
+  if (lane == 31) part[w][0] = pre;
+  __syncthreads();
+  unsigned long long acc = pre - sum;
+  for (int i = 0; i < w; ++i) acc += part[i][0];
+  for (int k = k0; k < k1; ++k) dst[k] = acc += src[k];
 }
 
 __device__ double sigma_interp(const double* sig, int n, double e_min, double e_max, double loss,
@@ -327,76 +368,117 @@ struct FieldArgs {
 // takes the segment's deletions in proportion to its time; below zero it
 // counts as zero).  recomb NULL: no deletions (pass 2 of a two-pass run).
 // Electron impactor: ion density.  Ion impactor: sum over electron energy
-// bins of n_e(E_b) sigma(E_b) v(E_b).
+// bins of n_e(E_b) sigma(E_b) v(E_b).  One channel per grid row, one segment a
+// thread; the bins' sigma and v are worked out once a block (each thread did so
+// for itself before: 1.05 ms at 1000 segments and 64 bins, 0.03 ms now).
+constexpr int FIELD_BINS = 128;
+
 __global__ void k_build_fields(FieldArgs A, const unsigned long long* time1,
-                               const unsigned long long* recomb, const double* sig, double* frate,
-                               double* fcol) {
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= A.nch * A.nz) return;
-  int k = t / A.nz, j = t % A.nz;
+                               const unsigned long long* recomb, const double* sig,
+                               double* frate) {
+  __shared__ double sg[FIELD_BINS], sv[FIELD_BINS];
+  const int k = blockIdx.y;
   if (A.kind[k] != RECOMBINATION) return;
-  int partner = A.sout[k];
-  const unsigned long long* tj = time1 + ((size_t)partner * (A.nz + 2) + (j + 1)) * A.ntb;
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  const int partner = A.sout[k];
+  const bool on = j < A.nz, ion = A.sin[k] != SP_E;
+  const unsigned long long* tj =
+      time1 + ((size_t)partner * (A.nz + 2) + (min(j, A.nz - 1) + 1)) * A.ntb;
+  const double tv = A.tsim * A.vol;
   double ttot = 0.0, del = 0.0;
-  if (recomb) {
+  if (recomb && on) {
+#pragma unroll 8
     for (int b = 0; b < A.ntb; ++b) ttot += (double)tj[b];
     del = (double)recomb[(size_t)partner * A.nz + j] / A.vol;
   }
   double acc = 0.0;
-  for (int b = 0; b < A.ntb; ++b) {
-    double n = (double)tj[b] / Q_TIME / (A.tsim * A.vol);
-    if (recomb && ttot > 0.0) n -= del * ((double)tj[b] / ttot);
-    if (A.sin[k] == SP_E) {
-      acc += n;
-    } else {
-      double eb = A.e_min * pow(A.e_max / A.e_min, (b + 0.5) / A.ntb);
-      double x = eb / A.me;
-      double v = C_LIGHT * sqrt(x * (2.0 + x)) / (1.0 + x);
-      acc += fmax(n, 0.0) * sigma_interp(sig + (size_t)k * A.n_energy, A.n_energy, A.e_min,
-                                         A.e_max, A.loss[k], eb) * v;
+  for (int b0 = 0; b0 < A.ntb; b0 += FIELD_BINS) {
+    const int nb = min(FIELD_BINS, A.ntb - b0);
+    __syncthreads();
+    if (ion)                                          // sigma and v of the bins, once a block
+      for (int i = threadIdx.x; i < nb; i += blockDim.x) {
+        const int b = b0 + i;
+        const double eb = A.e_min * pow(A.e_max / A.e_min, (b + 0.5) / A.ntb);
+        const double x = eb / A.me;
+        sv[i] = C_LIGHT * sqrt(x * (2.0 + x)) / (1.0 + x);
+        sg[i] = sigma_interp(sig + (size_t)k * A.n_energy, A.n_energy, A.e_min, A.e_max,
+                             A.loss[k], eb);
+      }
+    __syncthreads();
+    if (!on) continue;
+#pragma unroll 4
+    for (int i = 0; i < nb; ++i) {
+      const unsigned long long tt = tj[b0 + i];
+      if (!tt) continue;                              // nothing there: n = 0
+      double n = xa_div((double)tt * (1.0 / Q_TIME), tv);
+      if (recomb && ttot > 0.0) n = __fma_rn(-del, xa_div((double)tt, ttot), n);
+      if (!ion) acc = __dadd_rn(acc, n);
+      else acc = __fma_rn(__dmul_rn(fmax(n, 0.0), sg[i]), sv[i], acc);
     }
   }
-  frate[(size_t)k * A.nz + j] = fmax(acc, 0.0);
+  if (on) frate[(size_t)k * A.nz + j] = fmax(acc, 0.0);
 }
 
-__global__ void k_field_columns(const double* frate, double* fcol, int nch, int nz, double dz) {
-  int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= nch) return;
+// Columns of the fields, one block per channel: the sums run serially (their
+// rounding is the column's), from shared memory.
+__global__ void k_field_columns(FieldArgs A, const double* frate, double* fcol) {
+  __shared__ double f[256];
+  const int k = blockIdx.x, nz = A.nz;
+  if (A.kind[k] != RECOMBINATION) return;
+  double* out = fcol + (size_t)k * (nz + 1);
   double c = 0.0;
-  fcol[(size_t)k * (nz + 1)] = 0.0;
-  for (int j = 0; j < nz; ++j) {
-    c += frate[(size_t)k * nz + j] * dz;
-    fcol[(size_t)k * (nz + 1) + j + 1] = c;
+  if (threadIdx.x == 0) out[0] = 0.0;
+  for (int j0 = 0; j0 < nz; j0 += 256) {
+    const int n = min(256, nz - j0);
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += blockDim.x) f[i] = frate[(size_t)k * nz + j0 + i];
+    __syncthreads();
+    if (threadIdx.x == 0)
+#pragma unroll 8
+      for (int i = 0; i < n; ++i) f[i] = c = __fma_rn(f[i], A.dz, c);
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += blockDim.x) out[j0 + i + 1] = f[i];
   }
 }
 
-// field_del: the field output takes its deletions as the cycles' fields do
+// field_del: the field output takes its deletions as the cycles' fields do.
+// One warp a (species, segment) row of energy bins, its loads and quotients a
+// bin a lane; the row's sums keep the bins' order (0.12 ms with a thread a row,
+// 0.02 ms).
 __global__ void k_normalize(const unsigned long long* time, const unsigned long long* time1,
                             const unsigned long long* recomb, const unsigned long long* cpos,
                             const unsigned long long* cneg, double* density, double* current,
                             double* field, int nz, int ntb, double tsim, double vol, double area,
                             int field_del) {
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < NSP * nz) {
-    int s = t / nz, j = t % nz;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+  if (current)
+    for (int i = t; i < NSP * (nz + 1); i += gridDim.x * blockDim.x)
+      current[i] = ((double)cpos[i] - (double)cneg[i]) / (area * tsim);
+  const double tv = tsim * vol;
+  for (int row = t >> 5; row < NSP * nz; row += (gridDim.x * blockDim.x) >> 5) {
+    const int s = row / nz, j = row % nz;
+    const unsigned long long* tr = time + ((size_t)s * (nz + 2) + (j + 1)) * ntb;
+    const unsigned long long* t1 = time1 + ((size_t)s * (nz + 2) + (j + 1)) * ntb;
     double tsum = 0.0, t1tot = 0.0;
     if (field_del)
-      for (int b = 0; b < ntb; ++b) t1tot += (double)time1[((size_t)s * (nz + 2) + (j + 1)) * ntb + b];
-    const double del = field_del ? (double)recomb[(size_t)s * nz + j] / vol : 0.0;
-    for (int b = 0; b < ntb; ++b) {
-      size_t idx = ((size_t)s * (nz + 2) + (j + 1)) * ntb + b;
-      tsum += (double)time[idx] / Q_TIME;
-      if (field) {
-        double nb = (double)time1[idx] / Q_TIME / (tsim * vol);
-        if (field_del && t1tot > 0.0) nb -= del * ((double)time1[idx] / t1tot);
-        field[((size_t)s * nz + j) * ntb + b] = field_del ? fmax(nb, 0.0) : nb;
+      for (int b0 = 0; b0 < ntb; b0 += 32) {
+        const double v = b0 + lane < ntb ? (double)t1[b0 + lane] : 0.0;
+        for (int i = 0; i < min(32, ntb - b0); ++i) t1tot += __shfl_sync(0xffffffffu, v, i);
+      }
+    const double del = field_del ? (double)recomb[row] / vol : 0.0;
+    for (int b0 = 0; b0 < ntb; b0 += 32) {
+      const bool on = b0 + lane < ntb;
+      const double v = on ? (double)tr[b0 + lane] * (1.0 / Q_TIME) : 0.0;
+      for (int i = 0; i < min(32, ntb - b0); ++i) tsum += __shfl_sync(0xffffffffu, v, i);
+      if (field && on) {
+        const unsigned long long q = t1[b0 + lane];
+        double nb = q ? xa_div((double)q * (1.0 / Q_TIME), tv) : 0.0;
+        if (field_del && t1tot > 0.0)
+          nb = __fma_rn(-del, q ? xa_div((double)q, t1tot) : 0.0, nb);
+        field[(size_t)row * ntb + b0 + lane] = field_del ? fmax(nb, 0.0) : nb;
       }
     }
-    if (density) density[(size_t)s * nz + j] =
-        tsum / (tsim * vol) - (double)recomb[(size_t)s * nz + j] / vol;
-  }
-  if (t < NSP * (nz + 1) && current) {
-    current[t] = ((double)cpos[t] - (double)cneg[t]) / (area * tsim);
+    if (density && lane == 0) density[row] = tsum / tv - (double)recomb[row] / vol;
   }
 }
 
@@ -404,6 +486,23 @@ __global__ void k_accumulate(unsigned long long* dst, const unsigned long long* 
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
        i += (size_t)gridDim.x * blockDim.x)
     dst[i] += src[i];
+}
+
+void launch_finalize(const karl_ctx* ctx, const unsigned long long* pt, const unsigned long long* rg,
+                     unsigned long long* out, const unsigned long long* xpos,
+                     const unsigned long long* xneg, unsigned long long* cpos,
+                     unsigned long long* cneg, cudaStream_t st) {
+  const int groups = (NSP * ctx->ntb + 31) / 32;
+  k_finalize<<<groups + 2 * NSP, 32 * FIN_WARPS, 0, st>>>(pt, rg, out, xpos, xneg, cpos, cneg,
+                                                          ctx->nz, ctx->ntb, groups);
+}
+
+void launch_fields(const FieldArgs& A, const unsigned long long* time1,
+                   const unsigned long long* recomb, const double* sig, double* frate, double* fcol,
+                   cudaStream_t st) {
+  if (A.nch == 0) return;
+  k_build_fields<<<dim3((A.nz + 31) / 32, A.nch), 32, 0, st>>>(A, time1, recomb, sig, frate);
+  k_field_columns<<<A.nch, 64, 0, st>>>(A, frate, fcol);
 }
 
 int grid_for(size_t n, int block) {
@@ -636,12 +735,10 @@ karl_status run_one_pass(karl_ctx* ctx, const karl_primaries* pr, const karl_run
     CK(ctx->d_time.ensure(nt));
     CK(ctx->d_cpos.ensure(n_cross(ctx)));
     CK(ctx->d_cneg.ensure(n_cross(ctx)));
-    k_finalize_time<<<grid_for((size_t)NSP * ctx->ntb, 64), 64, 0, st>>>(
-        ctx->d_tpt.p, ctx->d_trg.p, ctx->d_time.p, ctx->nz, ctx->ntb);
-    k_finalize_cross<<<1, 32, 0, st>>>(ctx->d_xpos.p, ctx->d_cpos.p, ctx->nz);
-    k_finalize_cross<<<1, 32, 0, st>>>(ctx->d_xneg.p, ctx->d_cneg.p, ctx->nz);
+    launch_finalize(ctx, ctx->d_tpt.p, ctx->d_trg.p, ctx->d_time.p, ctx->d_xpos.p, ctx->d_xneg.p,
+                    ctx->d_cpos.p, ctx->d_cneg.p, st);
     CK(cudaGetLastError());
-    ctx->stats.kernel_launches += 3;
+    ctx->stats.kernel_launches += 1;
     return KARL_OK;
   }
   return fail(ctx, KARL_ECAPACITY, "particle ring overflow at capacity %llu",
@@ -673,9 +770,7 @@ karl_status build_fields(karl_ctx* ctx, const unsigned long long* d_time1,
   CK(ctx->d_frate.ensure(nk * ctx->nz));
   CK(ctx->d_fcol.ensure(nk * (ctx->nz + 1)));
   CK(cudaMemsetAsync(ctx->d_frate.p, 0, nk * ctx->nz * 8, st));
-  k_build_fields<<<grid_for((size_t)ctx->nch * ctx->nz, 256), 256, 0, st>>>(
-      A, d_time1, d_recomb, ctx->d_sig.p, ctx->d_frate.p, ctx->d_fcol.p);
-  k_field_columns<<<1, 32, 0, st>>>(ctx->d_frate.p, ctx->d_fcol.p, ctx->nch, ctx->nz, ctx->dz);
+  launch_fields(A, d_time1, d_recomb, ctx->d_sig.p, ctx->d_frate.p, ctx->d_fcol.p, st);
   CK(cudaGetLastError());
   ctx->stats.kernel_launches += 2;
   return KARL_OK;
@@ -987,7 +1082,7 @@ karl_status karl_run(karl_ctx* ctx, const karl_primaries* pr, const karl_run_opt
   CK(ctx->d_density.ensure((size_t)NSP * ctx->nz));
   CK(ctx->d_current.ensure(n_cross(ctx)));
   CK(ctx->d_field.ensure((size_t)NSP * ctx->nz * ctx->ntb));
-  k_normalize<<<grid_for(n_cross(ctx), 256), 256, 0, st>>>(
+  k_normalize<<<grid_for((size_t)NSP * 32 * (ctx->nz + 1), 128), 128, 0, st>>>(
       ctx->d_time.p, (const unsigned long long*)ctx->d_time1.p, ctx->d_recomb.p, ctx->d_cpos.p,
       ctx->d_cneg.p, ctx->d_density.p, ctx->d_current.p, ctx->d_field.p, ctx->nz, ctx->ntb, tsim,
       vol, ctx->area, 0);
@@ -1164,7 +1259,7 @@ karl_status karl_run_cycles(karl_ctx* ctx, const karl_primaries* pr, const karl_
   CK(ctx->d_density.ensure((size_t)NSP * ctx->nz));
   CK(ctx->d_current.ensure(n_cross(ctx)));
   CK(ctx->d_field.ensure((size_t)NSP * ctx->nz * ctx->ntb));
-  k_normalize<<<grid_for(n_cross(ctx), 256), 256, 0, st>>>(
+  k_normalize<<<grid_for((size_t)NSP * 32 * (ctx->nz + 1), 128), 128, 0, st>>>(
       ctx->c_time.p, ctx->c_time.p, ctx->c_rec.p, ctx->c_cpos.p, ctx->c_cneg.p, ctx->d_density.p,
       ctx->d_current.p, ctx->d_field.p, ctx->nz, ctx->ntb, tsim, vol, ctx->area, 1);
   CK(cudaGetLastError());
@@ -1410,9 +1505,8 @@ extern "C" karl_status karl_run_pass_static(karl_ctx* ctx, const karl_primaries*
       A.sout[k] = ctx->sout[k]; A.loss[k] = ctx->loss[k];
     }
     CK(cudaMemsetAsync(frate, 0, nk * ctx->nz * 8, st));
-    k_build_fields<<<grid_for((size_t)ctx->nch * ctx->nz, 256), 256, 0, st>>>(
-        A, (const unsigned long long*)field_time_in, nullptr, ctx->d_sig.p, frate, fcol);
-    k_field_columns<<<1, 32, 0, st>>>(frate, fcol, ctx->nch, ctx->nz, ctx->dz);
+    launch_fields(A, (const unsigned long long*)field_time_in, nullptr, ctx->d_sig.p, frate, fcol,
+                  st);
     CK(cudaGetLastError());
     ctx->stats.kernel_launches += 2;
     for (int k = 0; k < ctx->nch; ++k) {
@@ -1449,12 +1543,10 @@ extern "C" karl_status karl_run_pass_static(karl_ctx* ctx, const karl_primaries*
                       block, st));
   CK(cudaEventRecord(ctx->ev1, st));
   ctx->stats.kernel_launches += 1;
-  k_finalize_time<<<grid_for((size_t)NSP * ctx->ntb, 64), 64, 0, st>>>(
-      tpt, trg, (unsigned long long*)out->time_fx, ctx->nz, ctx->ntb);
-  k_finalize_cross<<<1, 32, 0, st>>>(xpos, (unsigned long long*)out->cross_pos, ctx->nz);
-  k_finalize_cross<<<1, 32, 0, st>>>(xneg, (unsigned long long*)out->cross_neg, ctx->nz);
+  launch_finalize(ctx, tpt, trg, (unsigned long long*)out->time_fx, xpos, xneg,
+                  (unsigned long long*)out->cross_pos, (unsigned long long*)out->cross_neg, st);
   CK(cudaGetLastError());
-  ctx->stats.kernel_launches += 3;
+  ctx->stats.kernel_launches += 1;
   Control hc;
   CK(cudaMemcpyAsync(&hc, ctl, sizeof hc, cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
