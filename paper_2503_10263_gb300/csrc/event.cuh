@@ -31,13 +31,29 @@ __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, 
 __device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
 __device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 
-// float <-> double of the FP32 form (the conversions: building them from the
-// bits measured slower there); identities for FP64
+// float <-> double of the FP32 form; identities for FP64.  GB300 converts on
+// the FP64 pipe, which the FP32 form keeps half busy (positions, time quanta),
+// so normal values are converted on the bits, rounded to nearest even.
 __device__ __forceinline__ double to_d(double x) { return x; }
-__device__ __forceinline__ double to_d(float x) { return (double)x; }
+__device__ __forceinline__ double to_d(float x) {
+  const int b = __float_as_int(x), m = b & 0x7fffffff;
+  if ((unsigned)(m - 0x00800000) >= 0x7f000000u) return (double)x;     // 0, subnormal, inf, NaN
+  return __hiloint2double((int)((unsigned)(b & 0x80000000) | (unsigned)((m >> 3) + (896 << 20))),
+                          m << 29);
+}
 template <class R> __device__ __forceinline__ R from_d(double x);
 template <> __device__ __forceinline__ double from_d<double>(double x) { return x; }
-template <> __device__ __forceinline__ float from_d<float>(double x) { return (float)x; }
+template <> __device__ __forceinline__ float from_d<float>(double x) {
+  const long long b = __double_as_longlong(x), u = b & 0x7fffffffffffffffLL;
+  if ((unsigned)((int)(u >> 52) - 897) >= 253u) return (float)x;       // outside [2^-126, 2^127)
+  const int r = (int)((u + 0x0fffffffLL + ((u >> 29) & 1)) >> 29) - (int)(896u << 23);
+  return __int_as_float(r | (int)(b >> 63 << 31));
+}
+// a parameter in the form's precision
+template <bool F32> __device__ __forceinline__ auto par(double d, float f) {
+  if constexpr (F32) return f;
+  else return d;
+}
 
 // out of line for the rare paths (the event itself takes them inline)
 static __device__ __noinline__ double div_call(double a, double b) { return xa_div(a, b); }
@@ -897,8 +913,8 @@ __device__ __forceinline__ void event(const Params& P, const Params& PS, const C
   o.flights += 1;
 
   // position of ln E among the table nodes (shared by both lookups)
-  const R le = T::lg(e * (R)P.inv_e_min);
-  const R lx = le * (R)P.inv_h;
+  const R le = T::lg(e * par<F32>(P.inv_e_min, P.inv_e_min_f));
+  const R lx = le * par<F32>(P.inv_h, P.inv_h_f);
   int ti;
   R tf;
   if constexpr (F32) ti = (int)floor(lx);
@@ -929,14 +945,15 @@ __device__ __forceinline__ void event(const Params& P, const Params& PS, const C
   // both from one reciprocal root, and the time quantum folded into the second
   const double amu = fabs(L.mu);
   const bool still = dzero(L.mu);
-  const R x = mul_rn(e, (R)P.inv_mass[s]);
+  const R x = mul_rn(e, par<F32>(P.inv_mass[s], P.inv_mass_f[s]));
+  const R muR = from_d<R>(L.mu);
   R inv_v;
   double inv_szq;                          // Q_T / (|mu| v): time units per metre along z
   if constexpr (F32) {
     inv_v = mul_rn(mul_rn((R)1 + x, (R)(1.0 / C_LIGHT)), T::rsq(mul_rn(x, (R)2 + x)));
-    const float amuf = (float)amu;
+    const float amuf = fabsf((float)muR);
     inv_szq = still ? 0.0
-            : amuf > 1e-20f ? (double)mul_rn(mul_rn(inv_v, __frcp_rn(amuf)), (float)Q_T)
+            : amuf > 1e-20f ? to_d(mul_rn(mul_rn(inv_v, __frcp_rn(amuf)), (float)Q_T))
                             : mul_rn((double)inv_v, Q_T / amu);  // keeps FP32 in range
   } else {
     const double m2 = still ? 1.0 : mul_rn(L.mu, L.mu);
@@ -997,7 +1014,7 @@ __device__ __forceinline__ void event(const Params& P, const Params& PS, const C
   // energy bin of the time tally
   int b = 0;
   if (P.ntb > 1) {
-    if constexpr (F32) b = (int)floor(le * (R)P.tb_scale);
+    if constexpr (F32) b = (int)floor(le * P.tb_scale_f);
     else b = floor_or_m1(le * P.tb_scale);
     b = b < 0 ? 0 : (b > P.ntb - 1 ? P.ntb - 1 : b);
   }
@@ -1055,7 +1072,7 @@ __device__ __forceinline__ void event(const Params& P, const Params& PS, const C
         ex = true;                          // no channel: straight to an end
       } else {
         double D;
-        if constexpr (F32) D = (double)mul_rn(mul_rn(tau, (R)amu), __frcp_rn(gas));
+        if constexpr (F32) D = to_d(mul_rn(mul_rn(tau, fabsf(muR)), __frcp_rn(gas)));
         else D = mul_rn(to_d(tau), amu) / gasd;
         const double c0 = fma_rn(tb.n(P, j0), L.z - tb.face(P, j0), tb.col(P, j0));
         tgt = up ? c0 + D : c0 - D;
@@ -1095,7 +1112,7 @@ __device__ __forceinline__ void event(const Params& P, const Params& PS, const C
       // check of G confirms it (the fields add little rate), and otherwise the
       // search goes on before it with G.
       gas_units = true;
-      const double ig = 1.0 / gasd;
+      const double ig = F32 ? xa_div(1.0, gasd) : 1.0 / gasd;
       rho0 = mul_rn(rc0, ig);
       rho1 = mul_rn(rc1, ig);
       auto gcol = [&](int k) -> double {
@@ -1300,8 +1317,8 @@ __device__ __forceinline__ void event(const Params& P, const Params& PS, const C
   } else if (kind == ELASTIC) {
     // CM polar angle (isotropic or tabulated at the lab energy, which is the
     // impact energy for a target at rest): lab polar angle and energy transfer
-    const R g = (R)P.gam[s];
-    const R g2 = (R)P.gam2[s];                 // 2 g
+    const R g = par<F32>(P.gam[s], P.gam_f[s]);
+    const R g2 = par<F32>(P.gam2[s], P.gam2_f[s]);   // 2 g
     R cchi, omc;                               // cos chi and 1 - cos chi
     const int ang = P.ch[k].ang;
     if (ang >= 0 && e >= (R)P.ang_thr[ang]) {
@@ -1317,14 +1334,15 @@ __device__ __forceinline__ void event(const Params& P, const Params& PS, const C
     const R ra = T::rsq(a);
     const R ct = mul_rn(cchi + g, ra);
     // energy given to the target, E - E' = E 2g(1 - cos chi)/(1+g)^2
-    const R de = mul_rn(mul_rn(mul_rn(e, g2), (R)1 - cchi), (R)P.inv_1pg2[s]);
+    const R de = mul_rn(mul_rn(mul_rn(e, g2), (R)1 - cchi),
+                        par<F32>(P.inv_1pg2[s], P.inv_1pg2_f[s]));
     long long rq = T::quant_de(de);
     if (rq > L.eq) rq = L.eq;
     o.recoil += (unsigned long long)rq;
     L.eq -= rq;
     // sin(theta_lab) sqrt(1 - mu^2) in one root: 1 - ct^2 = (1 - cchi^2) / a
     const R cphi = T::cpi(mul_rn((R)2, T::u(w[3])));
-    const R mu = from_d<R>(L.mu);
+    const R mu = muR;
     const R s2 = T::max0(mul_rn(fma_rn(-cchi, cchi, (R)1), fma_rn(-mu, mu, (R)1)));
     const R ss = mul_rn(F32 ? (R)sqrtf((float)s2) : (R)sqrt((double)s2), ra);
     L.mu = to_d(T::clamp1(fma_rn(mu, ct, mul_rn(ss, cphi))));

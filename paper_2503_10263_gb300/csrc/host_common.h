@@ -307,6 +307,15 @@ inline void fill_params(Params& P, const karl_geometry& g, const ModelInfo& m, i
     P.gam2[s] = 2.0 * P.gam[s];
     P.inv_1pg2[s] = 1.0 / ((1.0 + P.gam[s]) * (1.0 + P.gam[s]));
   }
+  P.inv_e_min_f = (float)P.inv_e_min;
+  P.inv_h_f = (float)P.inv_h;
+  P.tb_scale_f = (float)(g.n_tebins / std::log(m.e_max / m.e_min));
+  for (int s = 0; s < NSP; ++s) {
+    P.inv_mass_f[s] = (float)P.inv_mass[s];
+    P.gam_f[s] = (float)P.gam[s];
+    P.gam2_f[s] = (float)P.gam2[s];
+    P.inv_1pg2_f[s] = (float)P.inv_1pg2[s];
+  }
   P.target_mass = g.target_mass_ev;
   P.eps_ion = m.eps_ion;
   P.inv_eps_ion = 1.0 / m.eps_ion;

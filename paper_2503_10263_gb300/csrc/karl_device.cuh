@@ -105,6 +105,10 @@ struct Params {
   double gam[NSP];              // m / M_target
   double gam2[NSP];             // 2 m / M_target
   double inv_1pg2[NSP];         // 1 / (1 + m/M)^2
+  // FP32 copies for the precision form (a conversion in the event would take
+  // the FP64 pipe)
+  float inv_e_min_f, inv_h_f, tb_scale_f;
+  float inv_mass_f[NSP], gam_f[NSP], gam2_f[NSP], inv_1pg2_f[NSP];
   double target_mass, eps_ion, inv_eps_ion, kT;
   double drift_c;               // gas drift along +z in units of c (moving targets)
   double target_a;              // sqrt(kT / target mass): thermal velocity component, units of c
