@@ -104,31 +104,36 @@ constexpr float XA_TIE = 0.4995f;
 // place, and the second correction's error is below 2^-11 units.  q0's
 // significand must keep eight FP32 units from its binade's ends, so the
 // corrections (four of them at most) stay within it.  Two FP64 instructions.
-XA_FN double xa_div(double a, double b) {
+// xa_div_try clears ok instead of calling the IEEE division (its value is then
+// meaningless), for straight code with one test for many quotients and roots.
+XA_FN double xa_div_try(double a, double b, bool& ok) {
   const long long sa = xa_bits(a) & (long long)0x8000000000000000ULL;
   const long long ba = xa_bits(a) ^ sa, bb = xa_bits(b);
   const int ea = (int)(ba >> 52), eb = (int)(bb >> 52);      // eb negative with the sign bit
+  const double ma = xa_dbl((ba & XA_MANT) | XA_ONE), mb = xa_dbl((bb & XA_MANT) | XA_ONE);
+  const float r = xa_rcp(xa_top24(bb));
+  const float q0f = xa_fmul(xa_top24(ba), r);                // in (0.5, 2)
+  const int qm = xa_fbits(q0f) & 0x7fffff;
+  // 2^52 or 2^53: units of the last place in q0's binade
+  const float unit = xa_fbits(q0f) < 0x3f800000 ? 9007199254740992.0f : 4503599627370496.0f;
+  const float ru = xa_fmul(r, unit);
+  const double q0 = xa_from_f(q0f);
+  const double r0 = xa_fma(-q0, mb, ma);
+  const int n0 = xa_rint(xa_fmul(xa_trunc_f(r0), xa_fmul(ru, 0.0625f)));   // units of 16
+  const long long b1 = xa_bits(q0) + ((long long)n0 << 4);
+  const double r1 = xa_fma(-xa_dbl(b1), mb, ma);
+  const float c1 = xa_fmul(xa_trunc_f(r1), ru);
+  const int n1 = xa_rint(c1);
+  const float off = c1 - xa_float(n1);
   // magnitudes in (2^-500, 2^500): normal, and so is the quotient
-  if ((unsigned)(ea - 523) < 1000u && (unsigned)(eb - 523) < 1000u) {
-    const double ma = xa_dbl((ba & XA_MANT) | XA_ONE), mb = xa_dbl((bb & XA_MANT) | XA_ONE);
-    const float r = xa_rcp(xa_top24(bb));
-    const float q0f = xa_fmul(xa_top24(ba), r);              // in (0.5, 2)
-    const int qm = xa_fbits(q0f) & 0x7fffff;
-    // 2^52 or 2^53: units of the last place in q0's binade
-    const float unit = xa_fbits(q0f) < 0x3f800000 ? 9007199254740992.0f : 4503599627370496.0f;
-    const float ru = xa_fmul(r, unit);
-    const double q0 = xa_from_f(q0f);
-    const double r0 = xa_fma(-q0, mb, ma);
-    const int n0 = xa_rint(xa_fmul(xa_trunc_f(r0), xa_fmul(ru, 0.0625f)));   // units of 16
-    const long long b1 = xa_bits(q0) + ((long long)n0 << 4);
-    const double r1 = xa_fma(-xa_dbl(b1), mb, ma);
-    const float c1 = xa_fmul(xa_trunc_f(r1), ru);
-    const int n1 = xa_rint(c1);
-    const float off = c1 - xa_float(n1);
-    if ((unsigned)(qm - 8) < 0x7fffffu - 16u && off < XA_TIE && off > -XA_TIE)
-      return xa_dbl((b1 + n1 + ((long long)(ea - eb) << 52)) | sa);
-  }
-  return xa_ieee_div(a, b);
+  ok = ok && (unsigned)(ea - 523) < 1000u && (unsigned)(eb - 523) < 1000u &&
+       (unsigned)(qm - 8) < 0x7fffffu - 16u && off < XA_TIE && off > -XA_TIE;
+  return xa_dbl((b1 + n1 + ((long long)(ea - eb) << 52)) | sa);
+}
+XA_FN double xa_div(double a, double b) {
+  bool ok = true;
+  const double q = xa_div_try(a, b, ok);
+  return ok ? q : xa_ieee_div(a, b);
 }
 
 // sqrt(a), correctly rounded; the same scheme with m in [1, 4), a = m 4^k,
@@ -136,72 +141,69 @@ XA_FN double xa_div(double a, double b) {
 // and corrections residual x y/2 (the root's second-order term is in the
 // first one's relative error, 2^-20.9; the second one's is below 2^-11 units).
 // Two FP64 instructions.
-XA_FN double xa_sqrt(double a) {
+XA_FN double xa_sqrt_try(double a, bool& ok) {
   const long long ba = xa_bits(a);
   const int e = (int)(ba >> 52);
-  if ((unsigned)(e - 523) < 1000u) {
-    const int odd = (e & 1) ^ 1;                             // exponent e - 1023 odd
-    const long long bm = (ba & XA_MANT) | ((long long)(1023 + odd) << 52);
-    const double m = xa_dbl(bm);
-    const float mf = xa_flt((xa_fbits(xa_top24(ba))) + (odd << 23));
-    const float y = xa_rsqrt(mf);
-    const float g0f = xa_fmul(mf, y);                        // in [1, 2)
-    const int gm = xa_fbits(g0f) & 0x7fffff;
-    const float yu = xa_fmul(y, 2251799813685248.0f);        // y/2 x 2^52
-    const double g0 = xa_from_f(g0f);
-    const double r0 = xa_fma(-g0, g0, m);
-    const int n0 = xa_rint(xa_fmul(xa_trunc_f(r0), xa_fmul(yu, 0.0625f)));
-    const long long b1 = xa_bits(g0) + ((long long)n0 << 4);
-    const double g1 = xa_dbl(b1);
-    const double r1 = xa_fma(-g1, g1, m);
-    const float c1 = xa_fmul(xa_trunc_f(r1), yu);
-    const int n1 = xa_rint(c1);
-    const float off = c1 - xa_float(n1);
-    if (g0f >= 1.0f && (unsigned)(gm - 8) < 0x7fffffu - 16u && off < XA_TIE && off > -XA_TIE)
-      return xa_dbl(b1 + n1 + ((long long)((e - odd - 1023) / 2) << 52));
-  }
-  return xa_ieee_sqrt(a);
+  const int odd = (e & 1) ^ 1;                               // exponent e - 1023 odd
+  const double m = xa_dbl((ba & XA_MANT) | ((long long)(1023 + odd) << 52));
+  const float mf = xa_flt((xa_fbits(xa_top24(ba))) + (odd << 23));
+  const float y = xa_rsqrt(mf);
+  const float g0f = xa_fmul(mf, y);                          // in [1, 2)
+  const int gm = xa_fbits(g0f) & 0x7fffff;
+  const float yu = xa_fmul(y, 2251799813685248.0f);          // y/2 x 2^52
+  const double g0 = xa_from_f(g0f);
+  const double r0 = xa_fma(-g0, g0, m);
+  const int n0 = xa_rint(xa_fmul(xa_trunc_f(r0), xa_fmul(yu, 0.0625f)));
+  const long long b1 = xa_bits(g0) + ((long long)n0 << 4);
+  const double g1 = xa_dbl(b1);
+  const double r1 = xa_fma(-g1, g1, m);
+  const float c1 = xa_fmul(xa_trunc_f(r1), yu);
+  const int n1 = xa_rint(c1);
+  const float off = c1 - xa_float(n1);
+  ok = ok && (unsigned)(e - 523) < 1000u && g0f >= 1.0f &&
+       (unsigned)(gm - 8) < 0x7fffffu - 16u && off < XA_TIE && off > -XA_TIE;
+  return xa_dbl(b1 + n1 + ((long long)((e - odd - 1023) / 2) << 52));
+}
+XA_FN double xa_sqrt(double a) {
+  bool ok = true;
+  const double g = xa_sqrt_try(a, ok);
+  return ok ? g : xa_ieee_sqrt(a);
 }
 
-// k with 1 + x = 1 + k 2^-52 rounded to nearest even, for 0 <= x < 2^-25
-// (then k < 2^27): x's significand shifted right by 1023 - e places.
-XA_FN int xa_ulps_of_1p(double x) {
+// j with sqrt(RN(1 + x)) = 1 + j 2^-52, correctly rounded, for 0 <= x < 2^-25.
+// RN(1 + x) = 1 + k 2^-52 with k = x 2^52 rounded to nearest even, and its root
+// is, in units of 2^-52, k/2 - d with 0 < d = k^2 2^-55 (1 - ...) < 1/2 (d = 0
+// at k = 0): an even k gives k/2, an odd one, just below the midpoint, the
+// integer below.  So j = floor(k/2) = floor((x 2^52 + 1/2) / 2), ties included,
+// which the 31 upper bits of x's significand decide.  No FP64 instruction.
+XA_FN int xa_gamma_ulps(double x) {
   const long long b = xa_bits(x);
   const int s = 1023 - (int)(b >> 52);                       // 26 and up
-  if (s > 53) return 0;                                      // x 2^52 below one half
-  const long long m = (b & XA_MANT) | 0x0010000000000000LL;
-  const long long h = 1LL << (s - 1);
-  return (int)((m + h - 1 + ((m >> s) & 1)) >> s);
+  const unsigned m = ((unsigned)(b >> 22) & 0x3fffffffu) | 0x40000000u;   // significand >> 22
+  return s > 53 ? 0 : (int)((m + (1u << ((s - 23) & 31))) >> ((s - 22) & 31)) >> 1;
 }
 
-// sqrt(1 + k 2^-52), correctly rounded, is 1 + floor(k/2) 2^-52 for
-// 0 <= k < 2^27: in units of 2^-52 the root is k/2 - d with
-// 0 < d = k^2 2^-55 (1 - ...) < 1/2 (d = 0 at k = 0), so an even k rounds to
-// k/2 and an odd one, just below the midpoint, down.
-XA_FN int xa_sqrt_ulps(int k) { return k >> 1; }
-
-// a / (1 + j 2^-52), correctly rounded, for 0 <= j < 2^26 and a normal a,
-// by integers: with the significand A, the quotient is A - w,
-// w = A j / (2^52 + j) = w0 - w0 j 2^-52 + ..., w0 = A j 2^-52.  In units of
-// 2^-52, w's fraction is taken as frac(w0) - floor(w0) j, off by less than
-// 2^28; a fraction nearer to one half than that, or an A - w below 2^52,
-// goes to the IEEE division.  No FP64 instruction.
-XA_FN double xa_div_1p(double a, int j) {
-  if (j == 0) return a;
+// a / (1 + j 2^-52), correctly rounded, for 0 <= j < 2^20 and a normal a: with
+// the significand A = 2^52 a', the quotient is A - w, w = a' j (1 - j 2^-52 +
+// ...).  w is taken from the 31 upper fraction bits of a', off by at most
+// j 2^-31 for those and a' j^2 2^-52 <= j 2^-31 for the second order; if it is
+// nearer to a midpoint than twice that, or A - w is not in a's binade, ok is
+// cleared.  No FP64 instruction.
+XA_FN double xa_div_1p_try(double a, int j, bool& ok) {
   const long long ba = xa_bits(a);
-  const unsigned long long A = (unsigned long long)(ba & XA_MANT) | 0x0010000000000000ULL;
-  const unsigned long long p0 = (A & 0xffffffffULL) * (unsigned long long)j;
-  const unsigned long long p1 = (A >> 32) * (unsigned long long)j + (p0 >> 32);
-  const int w0 = (int)(p1 >> 20);                            // floor(A j 2^-52) < 2^27
-  const long long frac = (long long)(((p1 & 0xfffffULL) << 32) | (p0 & 0xffffffffULL));
-  const long long g = frac - (long long)w0 * j + (1LL << 51);
-  const long long n = w0 + (g >> 52);                        // w rounded to nearest
-  const long long rest = g & XA_MANT;
+  const unsigned a31 = ((unsigned)(ba >> 21) & 0x7fffffffu) | 0x80000000u;   // a' 2^31
+  const unsigned long long w = (unsigned long long)a31 * (unsigned)j + (1u << 30);
+  const long long n = (long long)(w >> 31);                  // w rounded
+  const unsigned rest = (unsigned)w & 0x7fffffffu, near = 4u * (unsigned)j + 4u;
   const int e = (int)(ba >> 52) & 0x7ff;
-  if (rest > (1LL << 28) && rest < (1LL << 52) - (1LL << 28) && (ba & XA_MANT) >= n &&
-      e > 0 && e < 0x7ff)
-    return xa_dbl(ba - n);
-  return xa_ieee_div(a, xa_dbl(XA_ONE + j));
+  ok = ok && (unsigned)j < (1u << 20) && (j == 0 || rest - near < 0x80000000u - 2 * near) &&
+       (ba & XA_MANT) >= n && e > 0 && e < 0x7ff;
+  return xa_dbl(ba - n);
+}
+XA_FN double xa_div_1p(double a, int j) {
+  bool ok = true;
+  const double q = xa_div_1p_try(a, j, ok);
+  return ok ? q : xa_ieee_div(a, xa_dbl(XA_ONE + j));
 }
 
 // x / 2 and 2 x on the exponent (exact); operands near the ends of the range

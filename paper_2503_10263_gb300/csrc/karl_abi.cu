@@ -8,7 +8,6 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <climits>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -1766,8 +1765,7 @@ extern "C" karl_status karl_run_orbit(karl_ctx* ctx, const karl_orbit* ob,
     if ((s = upload(ctx, ctx->o_bin2, b2.data(), b2.size(), st))) return s;
     O.bin2 = ctx->o_bin2.p;
     O.R2_lo = (float)(O.R2 * (1.0 - in));
-    // the smallest z of each segment floor(z inv_dz); every z below the
-    // second one's belongs to the first, every z from the last one's up to it
+    // the smallest z of each segment floor(z inv_dz) within [0, L]
     std::vector<long long> ze(nz + 1);
     for (size_t j = 1; j < nz; ++j) {
       double z = (double)j / O.inv_dz;
@@ -1775,8 +1773,9 @@ extern "C" karl_status karl_run_orbit(karl_ctx* ctx, const karl_orbit* ob,
       while (z * O.inv_dz < (double)j) z = std::nextafter(z, INFINITY);
       std::memcpy(&ze[j], &z, sizeof z);
     }
-    ze[0] = LLONG_MIN;
-    ze[nz] = LLONG_MAX;
+    ze[0] = 0;
+    std::memcpy(&ze[nz], &ctx->L, sizeof(double));
+    ze[nz] += 1;
     if ((s = upload(ctx, ctx->o_zedge, ze.data(), ze.size(), st))) return s;
     O.zedge = ctx->o_zedge.p;
     CK(cudaStreamSynchronize(st));        // the host tables above go out of scope

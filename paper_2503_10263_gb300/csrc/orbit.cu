@@ -99,14 +99,6 @@ __device__ __forceinline__ int seg_of(const Params& P, const OrbitDev& O, double
   return j < 0 ? 0 : (j > P.nz - 1 ? P.nz - 1 : j);
 }
 
-// segment of z, js if z lies between that segment's edges (integer compares;
-// the edges are the exact thresholds of seg_of)
-__device__ __forceinline__ int seg_near(const Params& P, const OrbitDev& O, double z, int js) {
-  const long long b = __double_as_longlong(z);
-  if (b >= __ldg(O.zedge + js) && b < __ldg(O.zedge + js + 1)) return js;
-  return seg_of(P, O, z);
-}
-
 // radial bin of (x, y), searched from the bin b (the particle's bin, or a
 // guess); the squared radii are non-negative, so they compare as integers
 __device__ __forceinline__ int rbin_from(const OrbitDev& O, double x, double y, int b) {
@@ -242,9 +234,59 @@ struct Flight {
   unsigned long long cn;
   double rate;                     // sum of sigma n (and sigma n^2) in segment cj
   int js, rs;                      // segment and radial bin of the particle
+  long long zlo, zhi;              // bits of z in segment js, within the tube: [zlo, zhi)
+  float rlo, rhi;                  // FP32 squared radii certain to lie in bin rs
+  double dt, h, hb;                // the species' step, q dt / 2m and h B
   unsigned redraw;                 // energy-bin stops since the last event
   unsigned long long w1, w2, w3;   // uniforms of the collision
 };
+
+// The bounds of the particle's cell (they only change with it).
+__device__ __forceinline__ void cell_bounds(const OrbitDev& O, Flight& F) {
+  F.zlo = __ldg(O.zedge + F.js);
+  F.zhi = __ldg(O.zedge + F.js + 1);
+  const float2 r = __ldg(O.bin2 + F.rs);
+  F.rlo = r.x;
+  F.rhi = r.y;
+}
+// One step's push and displacement.
+struct Step {
+  double unx, uny, unz, u2n;       // proper velocity after the step and its square
+  double dx, dy, dz, ds;           // displacement and its length
+};
+
+// Boris push: half electric kick, magnetic rotation, half kick.  TRY: straight
+// code that clears ok where a quotient or root could not be settled, or, with
+// SMALL, where x = (u/c)^2 is not below 2^-25 (ions up to 80 eV; there gamma =
+// 1 + j 2^-52 follows from x by integers, and so do the quotients by it).
+template <bool TRY, bool SMALL>
+__device__ __forceinline__ void boris(const OrbitDev& O, const Flight& F, double kx, double ky,
+                                      double kz, double umx, double umy, double umz, double xm,
+                                      Step& S, bool& ok) {
+  auto div = [&](double a, double b) { return TRY ? xa_div_try(a, b, ok) : xa_div(a, b); };
+  auto root = [&](double a) { return TRY ? xa_sqrt_try(a, ok) : xa_sqrt(a); };
+  double t;
+  if (SMALL) t = xa_div_1p_try(F.hb, xa_gamma_ulps(xm), ok);
+  else t = div(F.hb, root(1.0 + xm));
+  const double sf = div(xa_twice(t), 1.0 + t * t);
+  const double upx = umx + umy * t, upy = umy - umx * t;
+  S.unx = umx + upy * sf + kx;
+  S.uny = umy - upx * sf + ky;
+  S.unz = O.ez ? umz + kz : (dzero(umz) ? umz + F.h * 0.0 : umz);
+  S.u2n = S.unx * S.unx + S.uny * S.uny + S.unz * S.unz;
+  const double xn2 = S.u2n * INV_C2;
+  double sc;
+  if (SMALL) {
+    ok = ok && bits(xn2) < X_SMALL;
+    sc = xa_div_1p_try(F.dt, xa_gamma_ulps(xn2), ok);
+  } else {
+    sc = div(F.dt, root(1.0 + xn2));
+  }
+  S.dx = S.unx * sc;
+  S.dy = S.uny * sc;
+  S.dz = S.unz * sc;
+  S.ds = root(S.dx * S.dx + S.dy * S.dy + S.dz * S.dz);
+}
 
 // Start a flight; false if the particle cannot move (stalled, ended here).
 __device__ bool start_flight(const Params& P, const OrbitDev& O, OPart& Q, Flight& F) {
@@ -284,6 +326,10 @@ __device__ bool start_flight(const Params& P, const OrbitDev& O, OPart& Q, Fligh
   F.rate = 0.0;
   F.js = seg_of(P, O, Q.z);
   F.rs = rbin_of(O, Q.x, Q.y);
+  cell_bounds(O, F);
+  F.dt = O.dt[Q.sp];
+  F.h = O.h[Q.sp];
+  F.hb = O.hb[Q.sp];
   atomicAdd(O.ledger + OB_N_FLIGHT, 1ULL);
   return true;
 }
@@ -468,8 +514,7 @@ __global__ void __launch_bounds__(512, 1) orbit_kernel(const Params P, const Orb
     }
     const int s = Q.sp;
     const double m = P.mass[s];
-    const double dt = O.dt[s];
-    const double h = O.h[s];
+    const double dt = F.dt;
     if (F.step >= O.max_steps) {
       flush_run(P, O, s, F.cj, F.cr, F.cn, 0.0, dt);
       const double e = kinetic_u(Q.ux, Q.uy, Q.uz, m);
@@ -480,37 +525,48 @@ __global__ void __launch_bounds__(512, 1) orbit_kernel(const Params P, const Orb
     }
     F.step += 1;
     steps += 1;
-    // Boris push: half electric kick, magnetic rotation, half kick.  With
-    // x = (u/c)^2 below 2^-25 (ions up to 80 eV) gamma = 1 + j 2^-52 follows
-    // from x by integers, and so do the quotients by it.
-    const double ex = O.er * Q.x, ey = O.er * Q.y;
-    const double kx = h * ex, ky = h * ey;
+    const double kx = F.h * (O.er * Q.x), ky = F.h * (O.er * Q.y);
+    const double kz = O.ez ? F.h * O.ez[F.js] : 0.0;
     const double umx = Q.ux + kx, umy = Q.uy + ky;
-    double umz, kz = 0.0;
-    if (O.ez) {
-      kz = h * O.ez[F.js];
-      umz = Q.uz + kz;
-    } else {
-      umz = dzero(Q.uz) ? Q.uz + h * 0.0 : Q.uz;
-    }
+    const double umz = O.ez ? Q.uz + kz : (dzero(Q.uz) ? Q.uz + F.h * 0.0 : Q.uz);
     const double xm = (umx * umx + umy * umy + umz * umz) * INV_C2;
-    double t;
-    if (bits(xm) < X_SMALL) t = xa_div_1p(O.hb[s], xa_sqrt_ulps(xa_ulps_of_1p(xm)));
-    else t = xa_div(O.hb[s], xa_sqrt(1.0 + xm));
-    const double sf = xa_div(xa_twice(t), 1.0 + t * t);
-    const double upx = umx + umy * t, upy = umy - umx * t;
-    const double unx = umx + upy * sf + kx;
-    const double uny = umy - upx * sf + ky;
-    const double unz = O.ez ? umz + kz : (dzero(umz) ? umz + h * 0.0 : umz);
-    const double u2n = unx * unx + uny * uny + unz * unz;
-    const double xn2 = u2n * INV_C2;
-    double sc;
-    if (bits(xn2) < X_SMALL) sc = xa_div_1p(dt, xa_sqrt_ulps(xa_ulps_of_1p(xn2)));
-    else sc = xa_div(dt, xa_sqrt(1.0 + xn2));
-    const double dx = unx * sc, dy = uny * sc, dz = unz * sc;
-    const double ds = xa_sqrt(dx * dx + dy * dy + dz * dz);
+    Step S;
+    bool ok = true;
+    if (bits(xm) < X_SMALL) boris<true, true>(O, F, kx, ky, kz, umx, umy, umz, xm, S, ok);
+    else boris<true, false>(O, F, kx, ky, kz, umx, umy, umz, xm, S, ok);
+    if (!ok) boris<false, false>(O, F, kx, ky, kz, umx, umy, umz, xm, S, ok);
+    const double unx = S.unx, uny = S.uny, unz = S.unz, u2n = S.u2n;
+    const double dx = S.dx, dy = S.dy, dz = S.dz, ds = S.ds;
     const double hx = xa_half(dx), hy = xa_half(dy), hz = xa_half(dz);
-    const int jm = seg_near(P, O, Q.z + hz, F.js);
+    const double xn = Q.x + dx, yn = Q.y + dy, zn = Q.z + dz, zm = Q.z + hz;
+    const double tn = Q.t + dt;
+    // squared radii of the step's end and midpoint in FP32 (relative error
+    // below 2^-20, for the midpoint's sums while the half step is below r / 4):
+    // they decide wall and bin away from the edges
+    const float xe = xa_trunc_f(xn), ye = xa_trunc_f(yn);
+    const float re2 = xe * xe + ye * ye;
+    const float hxf = xa_trunc_f(hx), hyf = xa_trunc_f(hy);
+    const float xc = xa_trunc_f(Q.x) + hxf, yc = xa_trunc_f(Q.y) + hyf;
+    const float rc2 = xc * xc + yc * yc;
+    const bool far = 16.0f * (hxf * hxf + hyf * hyf) < rc2;
+    const bool rm_in = far && rc2 > F.rlo && rc2 < F.rhi, re_in = re2 > F.rlo && re2 < F.rhi;
+    const bool zm_in = bits(zm) >= F.zlo && bits(zm) < F.zhi;
+    const bool ze_in = bits(zn) >= F.zlo && bits(zn) < F.zhi;
+    // a step within its cell that ends no flight: the usual one
+    {
+      const double dtau = F.rate * ds, acc = F.acc + dtau;
+      if (rm_in && re_in && re2 < O.R2_lo && zm_in && ze_in && F.cj == F.js && F.cr == F.rs &&
+          bits(tn) < bits(P.max_life) && !(dpos(dtau) && bits(acc) >= bits(F.tau)) &&
+          bits(u2n) >= bits(F.u2lo) && bits(u2n) < bits(F.u2hi)) {
+        F.cn += 1;
+        Q.x = xn; Q.y = yn; Q.z = zn;
+        Q.t = tn;
+        F.acc = acc;
+        Q.ux = unx; Q.uy = uny; Q.uz = unz;
+        continue;
+      }
+    }
+    const int jm = zm_in ? F.js : seg_of(P, O, zm);
     if (jm != F.cj) {
       const double nm = P.nseg[jm];
       F.rate = F.s1 * nm + F.s3 * (nm * nm);
@@ -519,12 +575,6 @@ __global__ void __launch_bounds__(512, 1) orbit_kernel(const Params P, const Orb
     // the first of wall, z end, lifetime cap and collision within the step
     double fb = 1.0;
     int event = EV_NONE, end = -1;
-    const double xn = Q.x + dx, yn = Q.y + dy, zn = Q.z + dz;
-    // squared radii of the step's end and midpoint in FP32 (relative error
-    // below 2^-20): they decide wall and bin away from the edges
-    const float2 rb2 = __ldg(O.bin2 + F.rs);
-    const float xe = xa_trunc_f(xn), ye = xa_trunc_f(yn);
-    const float re2 = xe * xe + ye * ye;
     if (!(re2 < O.R2_lo) && bits(xn * xn + yn * yn) > bits(O.R2)) {
       const double a = dx * dx + dy * dy;
       const double b = Q.x * dx + Q.y * dy;
@@ -540,7 +590,7 @@ __global__ void __launch_bounds__(512, 1) orbit_kernel(const Params P, const Orb
       f = clamp01(f);
       if (event == EV_NONE ? f <= fb : f < fb) { fb = f; event = EV_EXIT; end = below ? 0 : 1; }
     }
-    if (bits(Q.t + dt) >= bits(P.max_life)) {
+    if (bits(tn) >= bits(P.max_life)) {
       const double f = clamp01((P.max_life - Q.t) / dt);
       if (event == EV_NONE ? f <= fb : f < fb) { fb = f; event = EV_CAP; }
     }
@@ -551,28 +601,23 @@ __global__ void __launch_bounds__(512, 1) orbit_kernel(const Params P, const Orb
     if (event == EV_NONE && (bits(u2n) < bits(F.u2lo) || bits(u2n) >= bits(F.u2hi)))
       event = EV_EBIN;
     if (event == EV_NONE || event == EV_EBIN) {
-      const float hxf = xa_trunc_f(hx), hyf = xa_trunc_f(hy);
-      const float xc = xa_trunc_f(Q.x) + hxf, yc = xa_trunc_f(Q.y) + hyf;
-      const float rc2 = xc * xc + yc * yc;
-      // (the sums' error stays below 2^-20 of r while the half step is below r / 4)
-      const bool far = 16.0f * (hxf * hxf + hyf * hyf) < rc2;
-      const int mr = far && rc2 > rb2.x && rc2 < rb2.y ? F.rs
-                                                       : rbin_from(O, Q.x + hx, Q.y + hy, F.rs);
+      const int mr = rm_in ? F.rs : rbin_from(O, Q.x + hx, Q.y + hy, F.rs);
       if (jm == F.cj && mr == F.cr) {
         F.cn += 1;
       } else {
         flush_run(P, O, s, F.cj, F.cr, F.cn, 0.0, dt);
         F.cj = jm; F.cr = mr; F.cn = 1;
       }
-      const int jb = seg_near(P, O, zn, F.js);
-      const int rb = re2 > rb2.x && re2 < rb2.y ? F.rs : rbin_from(O, xn, yn, F.rs);
+      const int jb = ze_in ? F.js : seg_of(P, O, zn);
+      const int rb = re_in ? F.rs : rbin_from(O, xn, yn, F.rs);
       if (jb != F.js || rb != F.rs) {
         crossings(P, O, s, F.js, F.rs, jb, rb);
         F.js = jb;
         F.rs = rb;
+        cell_bounds(O, F);
       }
       Q.x = xn; Q.y = yn; Q.z = zn;
-      Q.t += dt;
+      Q.t = tn;
       F.acc += dtau;
       Q.ux = unx; Q.uy = uny; Q.uz = unz;
       if (event == EV_NONE) continue;

@@ -44,7 +44,8 @@ struct OrbitDev {
   double r_scale;               // radial bins per metre (first guess of a bin)
   const double* edge2;          // [nr+1] squared radii of the radial bin edges
   const float2* bin2;           // [nr] FP32 squared radii certain to lie in the bin: (low, high)
-  const long long* zedge;       // [nz+1] bits of the smallest z in each segment (first: any)
+  const long long* zedge;       // [nz+1] bits of the smallest z in each segment; past the
+                                // last one those of the next number after L
   double er;                    // radial field per metre (V/m^2)
   double dt[NSP];               // Boris time step per species
   double h[NSP];                // q dt / 2m per species (m/s per V/m)

@@ -51,12 +51,13 @@ CHK int chk_one(uint64_t i) {
   double x = chk_from(((long long)(1023 - 26 - (int)(r3 % 60)) << 52) | (long long)(r1 >> 12));
   if (near == 1) x = (double)(2 * (int)(r2 % 100000) + 1) * 1.1102230246251565e-16;   // ties
   const double y = 1.0 + x;
-  const int k = xa_ulps_of_1p(x);
-  bad += xa_bits(y) - XA_ONE != k;
-  bad += xa_bits(xa_ieee_sqrt(y)) - XA_ONE != xa_sqrt_ulps(k);
-  bad += !chk_same(xa_div_1p(a, xa_sqrt_ulps(k)), xa_ieee_div(a, xa_ieee_sqrt(y)));
-  const int top = (1 << 27) - 1 - (int)(r2 & 0xffff);
-  bad += xa_bits(xa_ieee_sqrt(chk_from(XA_ONE + top))) - XA_ONE != xa_sqrt_ulps(top);
-  bad += !chk_same(xa_div_1p(a, top >> 1), xa_ieee_div(a, chk_from(XA_ONE + (top >> 1))));
+  const int j = xa_gamma_ulps(x);
+  bad += xa_bits(xa_ieee_sqrt(y)) - XA_ONE != j;
+  bad += !chk_same(xa_div_1p(a, j), xa_ieee_div(a, xa_ieee_sqrt(y)));
+  const double top = chk_from(((1023LL - 25) << 52) - 1 - (long long)(r2 & 0xffffffffffULL));
+  bad += xa_bits(xa_ieee_sqrt(1.0 + top)) - XA_ONE != xa_gamma_ulps(top);
+  const int jt = (int)(r3 >> 40) >> (r3 & 15);
+  bad += !chk_same(xa_div_1p(a, jt), xa_ieee_div(a, chk_from(XA_ONE + jt)));
+  bad += xa_gamma_ulps(0.0) != 0;
   return bad;
 }
