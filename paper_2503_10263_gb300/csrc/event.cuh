@@ -166,12 +166,15 @@ struct Lane {
   unsigned ev;                  // collisions so far = index of the next flight
   int sp;                       // species
   int j;                        // segment holding z (carried from the last flight)
-  int slot;                     // request slot (multi-request kernel; 0 otherwise)
+  int slot;                     // multi-request kernel: request slot, and SECOND in its second
+                                // pass; 0 otherwise
 };
+constexpr int SECOND = 1024;    // (slots are below it)
 
 // segment (20 bits) | species (2 bits) | request slot (10 bits) in one ring word
+// (the pass is the sign of the ring's time)
 __device__ __forceinline__ unsigned pack_sj(const Lane& p) {
-  return (unsigned)p.j | ((unsigned)p.sp << 20) | ((unsigned)p.slot << 22);
+  return (unsigned)p.j | ((unsigned)p.sp << 20) | ((unsigned)p.slot << 22);   // SECOND drops out
 }
 __device__ __forceinline__ void unpack_sj(unsigned w, Lane& p) {
   p.j = (int)(w & 0xfffffu);
@@ -244,7 +247,8 @@ __device__ __forceinline__ bool ring_put(const Ring& R, Control* ctl, unsigned l
     __nanosleep(64);
   }
   size_t i = pos & R.mask;
-  R.z[i] = p.z; R.eq[i] = p.eq; R.mu[i] = p.mu; R.node[i] = p.node; R.tal[i] = p.tal;
+  R.z[i] = p.z; R.eq[i] = p.eq; R.mu[i] = p.mu; R.node[i] = p.node;
+  R.tal[i] = p.slot & SECOND ? -p.tal : p.tal;   // (>= 0; its sign holds the request's pass)
   R.pid[i] = p.pid; R.ev[i] = p.ev; R.sj[i] = pack_sj(p);
   st_release(cell, pos + 1);
   return true;
@@ -263,9 +267,11 @@ __device__ __forceinline__ bool ring_get(const Ring& R, Control* ctl, unsigned l
     __nanosleep(32);
   }
   size_t i = pos & R.mask;
-  p.z = R.z[i]; p.eq = R.eq[i]; p.mu = R.mu[i]; p.node = R.node[i]; p.tal = R.tal[i];
+  p.z = R.z[i]; p.eq = R.eq[i]; p.mu = R.mu[i]; p.node = R.node[i];
+  p.tal = fabs(R.tal[i]);
   p.pid = R.pid[i]; p.ev = R.ev[i];
   unpack_sj(R.sj[i], p);
+  if (__double_as_longlong(R.tal[i]) < 0) p.slot |= SECOND;
   st_release(cell, pos + R.cap);
   return true;
 }
@@ -844,14 +850,14 @@ __device__ __noinline__ int select_per_channel(const Params& P, int s, long long
     for (int c = 0; c < nsc; ++c) {
       const int kk = P.sc[s][c];
       rtot = fma_rn((double)channel_coef<F32>(P, kk, s, eq, ti, tf, inv_v),
-                    field_kind(P.ch[kk].kind) ? P.frate[kk][jc] : nj, rtot);
+                    field_kind(P.ch[kk].kind) ? P.frate[kk][(size_t)jc * P.fstep] : nj, rtot);
     }
     const double target = mul_rn(u01d(w1), rtot);
     double cum = 0.0;
     for (int c = 0; c < nsc; ++c) {
       const int kk = P.sc[s][c];
       const double rk = mul_rn((double)channel_coef<F32>(P, kk, s, eq, ti, tf, inv_v),
-                               field_kind(P.ch[kk].kind) ? P.frate[kk][jc] : nj);
+                               field_kind(P.ch[kk].kind) ? P.frate[kk][(size_t)jc * P.fstep] : nj);
       if (!(rk > 0.0)) continue;
       last = c;
       cum += rk;
@@ -880,6 +886,18 @@ struct GlobalCols {
   __device__ __forceinline__ int ginv(const Params& P, int q) const { return P.ginv[q]; }
   __device__ __forceinline__ double fcol(const Params& P, int c, int k) const { return P.fcol[c][k]; }
   __device__ __forceinline__ double frate(const Params& P, int c, int j) const { return P.frate[c][j]; }
+};
+
+// The server's layout: one 32-byte record per face and segment, the field
+// tables as pairs of column and rate.
+struct RecordCols {
+  __device__ __forceinline__ double col(const Params& P, int k) const { return P.rec[4 * k]; }
+  __device__ __forceinline__ double face(const Params& P, int k) const { return P.rec[4 * k + 1]; }
+  __device__ __forceinline__ double n(const Params& P, int j) const { return P.rec[4 * j + 2]; }
+  __device__ __forceinline__ double invn(const Params& P, int j) const { return P.rec[4 * j + 3]; }
+  __device__ __forceinline__ int ginv(const Params& P, int q) const { return P.ginv[q]; }
+  __device__ __forceinline__ double fcol(const Params& P, int c, int k) const { return P.fcol[c][2 * k]; }
+  __device__ __forceinline__ double frate(const Params& P, int c, int j) const { return P.frate[c][2 * j]; }
 };
 
 // One event of the particle L.  A collision in a rare channel is left to the

@@ -124,7 +124,7 @@ inline bool xs_ok(const karl_xs* x) {
 // inverse density of each segment (0 without gas), and the inverse column on
 // nq even steps (a search bracket for the flights).
 struct ColumnTables {
-  std::vector<double> col, faces, invn;
+  std::vector<double> col, faces, invn, rec;
   std::vector<int> ginv;
   int nq = 0;
   double colmax = 0.0;
@@ -142,6 +142,13 @@ inline ColumnTables column_tables(const double* nseg, int nz, double length) {
   t.faces.resize(nz + 1);
   for (int k = 0; k < nz; ++k) t.faces[k] = (double)k * dz;
   t.faces[nz] = length;
+  t.rec.assign((size_t)4 * (nz + 1), 0.0);
+  for (int k = 0; k <= nz; ++k) {
+    double* r = t.rec.data() + (size_t)4 * k;
+    r[0] = t.col[k];
+    r[1] = t.faces[k];
+    if (k < nz) { r[2] = nseg[k]; r[3] = t.invn[k]; }
+  }
   t.colmax = t.col[nz];
   t.nq = t.colmax > 0 ? std::min(8192, std::max(256, nz)) : 0;
   t.ginv.assign(t.nq + 1, 0);
@@ -258,6 +265,7 @@ inline int leading_gas_channels(const ModelInfo& m, int s) {
 inline void fill_params(Params& P, const karl_geometry& g, const ModelInfo& m, int pass,
                         unsigned long long seed, int nq, double colmax) {
   std::memset(&P, 0, sizeof P);
+  P.fstep = 1;
   P.nz = g.n_zbins;
   P.L = g.length_m;
   P.dz = g.length_m / g.n_zbins;

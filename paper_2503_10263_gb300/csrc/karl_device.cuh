@@ -61,6 +61,11 @@ struct Params {
   const double* faces;     // [nz+1] face positions k*dz (face nz = L exactly)
   const int* ginv;         // [nq+1] largest face k with colgas[k] <= q * colmax / nq
   const double* invn;      // [nz] 1 / n_j (0 in a segment without gas)
+  // the same as one 32-byte record per face and the segment from it (column,
+  // position, density, inverse density): one memory sector for what a flight
+  // reads of a segment; multi-request kernel only
+  const double* rec;       // [nz+1][4]
+  int fstep;               // stride of the field tables below (2: pairs of column and rate)
   int nq;
   double nq_over_colmax;   // nq / colgas[nz] (0 if the column is empty)
   float nq_over_colmax_f;  // same in FP32 (search hints only)

@@ -116,7 +116,7 @@ __device__ void field_rates(const Params& P, const SlotDesc& d, int u, int lane)
         else acc = __fma_rn(__dmul_rn(n, sb), vb, acc);
       }
     }
-    if (j < nz) d.frate[(size_t)k * nz + j] = acc;
+    if (j < nz) d.fpair[((size_t)k * (nz + 1) + j) * 2 + 1] = acc;
   }
 }
 
@@ -124,17 +124,16 @@ __device__ void field_rates(const Params& P, const SlotDesc& d, int u, int lane)
 __device__ void field_columns(const Params& P, const SlotDesc& d, int lane) {
   const int nz = P.nz;
   if (lane >= P.nch || P.ch[lane].kind != RECOMBINATION) return;
-  const double* f = d.frate + (size_t)lane * nz;
-  double* out = d.fcol + (size_t)lane * (nz + 1);
+  double* f = d.fpair + (size_t)lane * (nz + 1) * 2;       // (column, rate) pairs
   double c = 0.0;
-  out[0] = 0.0;
+  f[0] = 0.0;
   for (int j = 0; j < nz; j += ROWS) {
     double a[ROWS];
 #pragma unroll
-    for (int i = 0; i < ROWS; ++i) a[i] = f[min(j + i, nz - 1)];
+    for (int i = 0; i < ROWS; ++i) a[i] = f[2 * min(j + i, nz - 1) + 1];
 #pragma unroll
     for (int i = 0; i < ROWS; ++i)
-      if (j + i < nz) out[j + i + 1] = c = __fma_rn(a[i], P.dz, c);
+      if (j + i < nz) f[2 * (j + i + 1)] = c = __fma_rn(a[i], P.dz, c);
   }
 }
 
@@ -335,9 +334,8 @@ __global__ void __launch_bounds__(256, 2) multi_kernel(SlotDesc* D, SlotCtl* C, 
   bool has = false;
   Lane L;
   L.slot = 0;
-  int lpass = 1;
   const Params* Pl = &D[0].P[0];
-  const GlobalCols cols{};
+  const RecordCols cols{};
   EventOut o;
   o.flights = o.colls = o.recoil = o.excit = 0;
   o.chan = -1;
@@ -367,12 +365,12 @@ __global__ void __launch_bounds__(256, 2) multi_kernel(SlotDesc* D, SlotCtl* C, 
   int credit = 0, T = step, quota = 32;
   bool drained = false, share = false, eager = false, idle = false;
 
-  // the lane's particle belongs to the current pass of its request
-  auto bind = [&](int s) {
-    lpass = ld_acquire_i(&C[s].pass);
-    lpass = lpass == 2 ? 2 : 1;
-    Pl = &D[s].P[lpass - 1];
-  };
+  // The lane's particle names its request and pass.  (The descriptor is the
+  // one its claim or its parent was bound to: a particle taken from the ring
+  // comes with an acquire of its cell.)
+  auto second = [&]() { return (L.slot & SECOND) != 0; };
+  auto slot_of = [&]() { return L.slot & (SECOND - 1); };
+  auto bind = [&]() { Pl = &D[slot_of()].P[second()]; };
   // per-lane sums belong to the request of the lane's particle: they go to
   // its ledger whenever the lane lets the particle go (death, park, hand-back)
   auto flush_sums = [&]() {
@@ -500,7 +498,7 @@ __global__ void __launch_bounds__(256, 2) multi_kernel(SlotDesc* D, SlotCtl* C, 
         if (rank < tr) {
           L = Rb.s[RB - r0 + rank];
           has = true;
-          bind(L.slot);
+          bind();
         }
       }
       __syncwarp();
@@ -520,7 +518,7 @@ __global__ void __launch_bounds__(256, 2) multi_kernel(SlotDesc* D, SlotCtl* C, 
           L = Q.s[top - 1 - rank];
           has = true;
           started += 1;
-          bind(L.slot);
+          bind();
         }
       }
       qleft = top - take;
@@ -628,9 +626,8 @@ __global__ void __launch_bounds__(256, 2) multi_kernel(SlotDesc* D, SlotCtl* C, 
           const unsigned long long idx = base + rank;
           if (src == 1) {
             has = ring_get(R, ctl, idx, L, deadline);
-            if (has) bind(L.slot);
+            if (has) bind();
           } else {
-            lpass = gpass;
             Pl = &D[gslot].P[gpass - 1];
             const Params& P = *Pl;
             L.z = P.pz[idx];
@@ -642,7 +639,7 @@ __global__ void __launch_bounds__(256, 2) multi_kernel(SlotDesc* D, SlotCtl* C, 
             L.ev = 0;
             L.pid = (unsigned long long)P.pid_offset + idx;
             L.j = segment_of(P, L.z);
-            L.slot = gslot;
+            L.slot = gslot | (gpass == 2 ? SECOND : 0);
             sadd(P.ledger + L_E_IN_PRIMARY, L.eq);
             sadd(P.ledger + L_BIRTHS + L.sp, 1);
             if (L.sp == SP_E && L.eq < P.ecut_q) {
@@ -694,7 +691,7 @@ __global__ void __launch_bounds__(256, 2) multi_kernel(SlotDesc* D, SlotCtl* C, 
         L = Rb.s[nr - 1 - rank];
         rk = Rb.ch[nr - 1 - rank];
         has = true;
-        bind(L.slot);
+        bind();
       }
       __syncwarp();                                // every parked slot has been read
       const int r0 = Rb.r;
@@ -734,7 +731,7 @@ __global__ void __launch_bounds__(256, 2) multi_kernel(SlotDesc* D, SlotCtl* C, 
         }
       }
       if (has && rk >= 0) {
-        port.slot_live = &C[L.slot].word[lpass - 1];
+        port.slot_live = &C[slot_of()].word[second()];
         Lane Mv = L;
         EventOut m;
         m.alive = true;
@@ -767,8 +764,8 @@ __global__ void __launch_bounds__(256, 2) multi_kernel(SlotDesc* D, SlotCtl* C, 
         flush_sums();
         __threadfence();                          // its tallies before its death
         const unsigned long long o2 =
-            atomicAdd(&C[L.slot].word[lpass - 1], (unsigned long long)0 - 1ULL);
-        if (pass_emptied(o2, 1ULL, D[L.slot].n_prim)) { trigB = 1; tslotB = L.slot; tpassB = lpass; }
+            atomicAdd(&C[slot_of()].word[second()], (unsigned long long)0 - 1ULL);
+        if (pass_emptied(o2, 1ULL, D[slot_of()].n_prim)) { trigB = 1; tslotB = slot_of(); tpassB = second() ? 2 : 1; }
       }
       credit += __popc(__ballot_sync(FULL, died)) - (qtop - qleft);
       if (credit < 0) {

@@ -64,8 +64,7 @@ struct SlotDesc {
   int pad0;
   long long n_prim;
   unsigned long long* time1;             // [3][nz+2][ntb] pass-1 time (target fields)
-  double* frate;                         // [nch][nz]
-  double* fcol;                          // [nch][nz+1]
+  double* fpair;                         // [nch][nz+1][2] field column and rate
   unsigned long long* time_out;          // [3][nz+2][ntb] time of the last pass
   unsigned long long* cpos_out;          // [3][nz+1]
   unsigned long long* cneg_out;          // [3][nz+1]

@@ -108,7 +108,7 @@ struct Request {
   int n_passes = 1;
   karl_tallies out;
   ColumnTables tabs;
-  std::vector<double> n2, col2;      // three-body clustering field (empty if unused)
+  std::vector<double> pair2;         // three-body clustering field, (column, rate) pairs
   // device pointers of the final pass and of the outputs, for collection
   unsigned long long *spec = nullptr, *rec = nullptr, *led = nullptr, *chan = nullptr;
   unsigned long long* led1 = nullptr;   // pass-1 ledger of a two-pass request, else NULL
@@ -207,11 +207,11 @@ cudaError_t zero_by_copy(const karl_server* srv, void* dst, size_t bytes, cudaSt
 size_t footprint(const Sizes& z) {
   size_t b = 0;
   b += 3 * up(z.n * 8) + up(z.n);                                   // primaries
-  b += 2 * up(z.nz * 8) + 2 * up((z.nz + 1) * 8) + up((z.nq + 1) * 4);  // tables
+  b += up(z.nz * 8) + up((z.nz + 1) * 32) + up((z.nq + 1) * 4);     // tables
   const size_t tallies = up(z.nspec * 8) + 2 * up(z.nt * 8) + 2 * up(z.cross_rg * 8) +
                          up(z.rec * 8) + up(LEDGER * 8) + up(MAXCH * 8);
   b += 2 * tallies;                                                 // both passes
-  b += up(z.nch * z.nz * 8) + up(z.nch * (z.nz + 1) * 8) + up(z.nt * 8);  // fields, time1
+  b += up(z.nch * (z.nz + 1) * 16) + up(z.nt * 8);                  // fields, time1
   b += up(z.nt * 8) + 3 * up(z.cross * 8) + up((size_t)NSP * z.nz * z.ntb * 8) +
        up((size_t)NSP * z.nz * 8);                                   // outputs
   return b;
@@ -272,9 +272,7 @@ karl_status admit(karl_server* srv, Request& r) {
   double* pmu = (double*)take(z.n * 8);
   uint8_t* psp = (uint8_t*)take(z.n);
   double* nseg = (double*)take(z.nz * 8);
-  double* invn = (double*)take(z.nz * 8);
-  double* col = (double*)take((z.nz + 1) * 8);
-  double* faces = (double*)take((z.nz + 1) * 8);
+  double* rec = (double*)take((z.nz + 1) * 32);
   int* ginv = (int*)take((z.nq + 1) * 4);
   char* tally0 = p;
   struct PassBufs {
@@ -291,8 +289,7 @@ karl_status admit(karl_server* srv, Request& r) {
     pb[k].chan = (unsigned long long*)take(MAXCH * 8);
   }
   const size_t tally_bytes = (size_t)(p - tally0);
-  double* frate = (double*)take(z.nch * z.nz * 8);
-  double* fcol = (double*)take(z.nch * (z.nz + 1) * 8);
+  double* fpair = (double*)take(z.nch * (z.nz + 1) * 16);
   unsigned long long* time1 = (unsigned long long*)take(z.nt * 8);
   r.time_out = (unsigned long long*)take(z.nt * 8);
   r.cpos = (unsigned long long*)take(z.cross * 8);
@@ -312,16 +309,12 @@ karl_status admit(karl_server* srv, Request& r) {
     SCK(cudaMemcpyAsync(psp, r.sp.data(), z.n, cudaMemcpyHostToDevice, cs));
   }
   SCK(cudaMemcpyAsync(nseg, r.nseg.data(), z.nz * 8, cudaMemcpyHostToDevice, cs));
-  SCK(cudaMemcpyAsync(invn, r.tabs.invn.data(), z.nz * 8, cudaMemcpyHostToDevice, cs));
-  SCK(cudaMemcpyAsync(col, r.tabs.col.data(), (z.nz + 1) * 8, cudaMemcpyHostToDevice, cs));
-  SCK(cudaMemcpyAsync(faces, r.tabs.faces.data(), (z.nz + 1) * 8, cudaMemcpyHostToDevice, cs));
+  SCK(cudaMemcpyAsync(rec, r.tabs.rec.data(), (z.nz + 1) * 32, cudaMemcpyHostToDevice, cs));
   SCK(cudaMemcpyAsync(ginv, r.tabs.ginv.data(), (z.nq + 1) * 4, cudaMemcpyHostToDevice, cs));
   SCK(zero_by_copy(srv, tally0, tally_bytes, cs));
   for (int c = 0; c < srv->model.nch; ++c)
     if (srv->model.kind[c] == CLUSTERING3) {
-      SCK(cudaMemcpyAsync(frate + (size_t)c * z.nz, r.n2.data(), z.nz * 8,
-                          cudaMemcpyHostToDevice, cs));
-      SCK(cudaMemcpyAsync(fcol + (size_t)c * (z.nz + 1), r.col2.data(), (z.nz + 1) * 8,
+      SCK(cudaMemcpyAsync(fpair + (size_t)c * (z.nz + 1) * 2, r.pair2.data(), (z.nz + 1) * 16,
                           cudaMemcpyHostToDevice, cs));
     }
   // descriptor
@@ -332,12 +325,11 @@ karl_status admit(karl_server* srv, Request& r) {
     Params& P = d.P[k];
     fill_params(P, r.g, srv->model, k + 1, r.seed, r.tabs.nq, r.tabs.colmax);
     P.nseg = nseg;
-    P.colgas = col;
-    P.faces = faces;
+    P.rec = rec;
+    P.fstep = 2;
     P.ginv = r.tabs.nq > 0 ? ginv : nullptr;
     P.sig = srv->d_sig_t;
     P.sigf = srv->d_sigf;
-    P.invn = invn;
     P.cum = srv->d_cum;
     P.cumf = srv->d_cumf;
     P.mixed = srv->d_mixed;
@@ -359,15 +351,14 @@ karl_status admit(karl_server* srv, Request& r) {
     P.per_primary = nullptr;
     for (int c = 0; c < srv->model.nch; ++c)
       if ((k == 1 && srv->model.kind[c] == RECOMBINATION) || srv->model.kind[c] == CLUSTERING3) {
-        P.frate[c] = frate + (size_t)c * z.nz;
-        P.fcol[c] = fcol + (size_t)c * (z.nz + 1);
+        P.fcol[c] = fpair + (size_t)c * (z.nz + 1) * 2;
+        P.frate[c] = P.fcol[c] + 1;
       }
   }
   d.n_passes = final_pass;
   d.n_prim = (long long)z.n;
   d.time1 = time1;
-  d.frate = frate;
-  d.fcol = fcol;
+  d.fpair = fpair;
   d.time_out = r.time_out;
   d.cpos_out = r.cpos;
   d.cneg_out = r.cneg;
@@ -774,7 +765,15 @@ karl_status karl_server_submit(karl_server* srv, const karl_geometry* g, const k
     r.sp.assign(pr->species, pr->species + pr->n);
     bool three_body = false;
     for (int c = 0; c < srv->model.nch; ++c) three_body |= srv->model.kind[c] == CLUSTERING3;
-    if (three_body) square_column(r.nseg.data(), g->n_zbins, g->length_m, r.n2, r.col2);
+    if (three_body) {
+      std::vector<double> n2, col2;
+      square_column(r.nseg.data(), g->n_zbins, g->length_m, n2, col2);
+      r.pair2.assign(2 * col2.size(), 0.0);
+      for (size_t k = 0; k < col2.size(); ++k) {
+        r.pair2[2 * k] = col2[k];
+        if (k < n2.size()) r.pair2[2 * k + 1] = n2[k];
+      }
+    }
   } catch (...) {
     return sfail(srv, KARL_ENOMEM, "host copy of the request");
   }
