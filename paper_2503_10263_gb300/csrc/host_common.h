@@ -24,6 +24,17 @@ struct TraceRange {
   TraceRange& operator=(const TraceRange&) = delete;
 };
 
+// Writes one byte of each page of an output buffer (the byte that is there).
+// A device-to-host copy into pages that no one has touched yet takes
+// their faults from the device's side: 3.5 ms more for 5 MB of fresh arrays
+// than for touched ones, which the host touches in 0.05 ms, and while the
+// device works.
+inline void touch_pages(void* p, size_t bytes) {
+  if (!p) return;
+  volatile unsigned char* c = (volatile unsigned char*)p;
+  for (size_t i = 0; i < bytes; i += 4096) c[i] = c[i];
+}
+
 constexpr double HOST_Q_ENERGY = 16777216.0;    // 2^24 units per eV
 constexpr double HOST_KB_EV = 8.617333262e-5;   // Boltzmann constant, eV/K
 

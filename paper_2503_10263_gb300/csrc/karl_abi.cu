@@ -207,6 +207,7 @@ struct karl_ctx {
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   karl_run_stats stats;
   std::string err;
+  std::vector<std::pair<void*, size_t>> touch;   // host outputs to touch while the next pass runs
   // every device buffer of the context
   template <class F>
   void each_buf(F f) {
@@ -696,6 +697,8 @@ karl_status run_one_pass(karl_ctx* ctx, const karl_primaries* pr, const karl_run
     CK(launch_transport(f32, P, R, ctx->d_ctl, ctx->d_cancel,
                         (unsigned long long)(timeout * 1e9), grid, block, st));
     CK(cudaEventRecord(ctx->ev1, st));
+    for (const auto& t : ctx->touch) touch_pages(t.first, t.second);
+    ctx->touch.clear();
     Control hc;
     CK(cudaMemcpyAsync(&hc, ctx->d_ctl, sizeof hc, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
@@ -781,6 +784,21 @@ karl_status copy_out(karl_ctx* ctx, void* dst, const void* src, size_t bytes, bo
   CK(cudaMemcpyAsync(dst, src, bytes, dst_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
                      st));
   return KARL_OK;
+}
+
+// The host outputs of a whole run, to be touched while its first pass runs.
+void touch_outputs(karl_ctx* ctx, const karl_tallies* out, size_t n) {
+  ctx->touch.clear();
+  if (out->on_device) return;
+  try {
+    ctx->touch = {{out->spectrum, n_spec(ctx) * 8}, {out->time_fx, n_time(ctx) * 8},
+                  {out->cross_pos, n_cross(ctx) * 8}, {out->cross_neg, n_cross(ctx) * 8},
+                  {out->recomb, n_recomb(ctx) * 8}, {out->per_primary, n * 8},
+                  {out->density, (size_t)NSP * ctx->nz * 8}, {out->current, n_cross(ctx) * 8},
+                  {out->field, (size_t)NSP * ctx->nz * ctx->ntb * 8}};
+  } catch (...) {
+    ctx->touch.clear();                          // (only a matter of speed)
+  }
 }
 
 karl_status check_opts(karl_ctx* ctx, const karl_run_opts* o) {
@@ -1056,6 +1074,7 @@ karl_status karl_run(karl_ctx* ctx, const karl_primaries* pr, const karl_run_opt
   s = stage_primaries(ctx, pr, st, &pz, &pe, &pmu, &psp);
   if (s) return s;
   bool pp = out->per_primary != nullptr && pr->n > 0;
+  touch_outputs(ctx, out, (size_t)pr->n);
   s = run_one_pass(ctx, pr, o, 1, pz, pe, pmu, psp, pp, st);
   if (s) return s;
   size_t nt = n_time(ctx);
@@ -1212,6 +1231,7 @@ karl_status karl_run_cycles(karl_ctx* ctx, const karl_primaries* pr, const karl_
     CK(cudaMemsetAsync(x.cum->p, 0, x.n * 8, st));
   }
   if (pp) CK(ctx->c_pp.ensure(nn));
+  touch_outputs(ctx, out, (size_t)pr->n);
   double kms = 0.0;
   int64_t colls = 0, flights = 0, parts = 0;
   const int64_t n = pr->n;

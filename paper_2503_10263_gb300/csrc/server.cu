@@ -415,7 +415,16 @@ karl_status admit(karl_server* srv, Request& r) {
   srv->seq += 1;
   r.state = REQ_ADMITTED;
   srv->stats.admitted += 1;
-  if (!srv->running) return launch(srv);
+  if (!srv->running) {
+    const karl_status st = launch(srv);
+    if (st) return st;
+  }
+  // the caller's buffers, while the request runs
+  const karl_tallies& t = r.out;
+  touch_pages(t.spectrum, z.nspec * 8);
+  touch_pages(t.time_fx, z.nt * 8);
+  touch_pages(t.density, (size_t)NSP * z.nz * 8);
+  touch_pages(t.field, (size_t)NSP * z.nz * z.ntb * 8);
   return KARL_OK;
 }
 
