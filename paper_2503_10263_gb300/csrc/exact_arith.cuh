@@ -174,13 +174,38 @@ XA_FN double xa_sqrt(double a) {
 // RN(1 + x) = 1 + k 2^-52 with k = x 2^52 rounded to nearest even, and its root
 // is, in units of 2^-52, k/2 - d with 0 < d = k^2 2^-55 (1 - ...) < 1/2 (d = 0
 // at k = 0): an even k gives k/2, an odd one, just below the midpoint, the
-// integer below.  So j = floor(k/2) = floor((x 2^52 + 1/2) / 2), ties included,
-// which the 31 upper bits of x's significand decide.  No FP64 instruction.
-XA_FN int xa_gamma_ulps(double x) {
-  const long long b = xa_bits(x);
-  const int s = 1023 - (int)(b >> 52);                       // 26 and up
-  const unsigned m = ((unsigned)(b >> 22) & 0x3fffffffu) | 0x40000000u;   // significand >> 22
-  return s > 53 ? 0 : (int)((m + (1u << ((s - 23) & 31))) >> ((s - 22) & 31)) >> 1;
+// integer below.  So j = floor(k/2) = floor((x 2^52 + 1/2) / 2), ties included.
+// For x = RN(RN(RN(RN(ux^2) + RN(uy^2)) + RN(uz^2)) / c^2), gamma of a proper
+// velocity of components below 2^14 m/s, it comes from 30-bit fixed-point
+// components: their squares' sum S (an integer, rounded components: relative
+// error below 2^-26) times 2^52 / c^2 gives x 2^52 with the error of S; where
+// that reaches an integer that floor((x 2^52 + 1/2) / 2) turns on, or a
+// component is too large, ok is cleared.  (The FP64 chain's own roundings are
+// below 2^-50.)  No FP64 instruction, against six for the chain.
+XA_FN unsigned long long xa_mulhi(unsigned long long a, unsigned long long b) {
+#ifdef __CUDACC__
+  return __umul64hi(a, b);
+#else
+  return (unsigned long long)(((unsigned __int128)a * b) >> 64);
+#endif
+}
+XA_FN int xa_gamma_ulps3(double ux, double uy, double uz, bool& ok) {
+  const long long bx = xa_bits(ux), by = xa_bits(uy), bz = xa_bits(uz);
+  const int ex = (int)(bx >> 52) & 0x7ff, ey = (int)(by >> 52) & 0x7ff, ez = (int)(bz >> 52) & 0x7ff;
+  int em = ex > ey ? ex : ey;
+  em = em > ez ? em : ez;
+  // components in units of 2^(em - 1023 - 29), below 2^30, rounded
+  const unsigned long long fx = ((((unsigned)(bx >> 21) | 0x80000000u) >> (em - ex > 30 ? 31 : em - ex + 1)) + 1) >> 1;
+  const unsigned long long fy = ((((unsigned)(by >> 21) | 0x80000000u) >> (em - ey > 30 ? 31 : em - ey + 1)) + 1) >> 1;
+  const unsigned long long fz = ((((unsigned)(bz >> 21) | 0x80000000u) >> (em - ez > 30 ? 31 : em - ez + 1)) + 1) >> 1;
+  const unsigned long long S = fx * fx + fy * fy + fz * fz;
+  // (2^56 / c^2) 2^64, rounded
+  const unsigned long long hi = xa_mulhi(S, 0xCD3F69CF4136CC8FULL);
+  const int s = 4 - 2 * (em - 1023 - 29);                    // x 2^52 = hi 2^-s
+  const unsigned long long A = hi + (1ULL << ((s - 1) & 63)), mask = (2ULL << (s & 63)) - 1;
+  const unsigned long long rem = A & mask, err = (hi >> 24) + 16;
+  ok = ok && em <= 1036 && s < 61 && rem > err && rem < mask - err;
+  return (int)(A >> ((s + 1) & 63));
 }
 
 // a / (1 + j 2^-52), correctly rounded, for 0 <= j < 2^20 and a normal a: with

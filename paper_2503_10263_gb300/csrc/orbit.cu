@@ -42,7 +42,8 @@ namespace {
 enum { EV_NONE = 0, EV_WALL = 1, EV_EXIT = 2, EV_CAP = 3, EV_COLL = 4, EV_EBIN = 5 };
 constexpr int DOM_REDRAW = 3;          // optical depths drawn anew after an energy-bin stop
 constexpr double INV_C2 = 1.0 / (C_LIGHT * C_LIGHT);
-constexpr long long X_SMALL = 0x3e60000000000000LL;   // 2^-25
+constexpr long long U_SMALL = 0x40d0000000000000LL;   // 2^14 m/s
+constexpr long long ABS = 0x7fffffffffffffffLL;
 
 // Comparisons of the step's tests on the bits of the doubles (integer
 // operations, the same outcomes as the floating-point compares for numbers:
@@ -229,6 +230,8 @@ __device__ void crossings(const Params& P, const OrbitDev& O, int s, int ja, int
 struct Flight {
   double tau, acc, e0, s1, s3;
   double u2lo, u2hi;               // the flight's energy bin as bounds on u^2
+  bool binned;                     // either is finite
+  bool small;                      // no component of u reaches 2^14 m/s (as last looked at)
   unsigned long long step;
   int cj, cr;                      // cell of the current run of steps
   unsigned long long cn;
@@ -240,6 +243,11 @@ struct Flight {
   unsigned redraw;                 // energy-bin stops since the last event
   unsigned long long w1, w2, w3;   // uniforms of the collision
 };
+
+// No component reaches U_SMALL.
+__device__ __forceinline__ bool slow(double ux, double uy, double uz) {
+  return max(max(bits(ux) & ABS, bits(uy) & ABS), bits(uz) & ABS) < U_SMALL;
+}
 
 // The bounds of the particle's cell (they only change with it).
 __device__ __forceinline__ void cell_bounds(const OrbitDev& O, Flight& F) {
@@ -256,32 +264,28 @@ struct Step {
 };
 
 // Boris push: half electric kick, magnetic rotation, half kick.  TRY: straight
-// code that clears ok where a quotient or root could not be settled, or, with
-// SMALL, where x = (u/c)^2 is not below 2^-25 (ions up to 80 eV; there gamma =
-// 1 + j 2^-52 follows from x by integers, and so do the quotients by it).
+// code that clears ok where a quotient or root could not be settled.  SMALL:
+// components below 2^14 m/s (thermal ions), where gamma = 1 + j 2^-52 follows
+// from them by integers, and so do the quotients by it.
 template <bool TRY, bool SMALL>
 __device__ __forceinline__ void boris(const OrbitDev& O, const Flight& F, double kx, double ky,
-                                      double kz, double umx, double umy, double umz, double xm,
-                                      Step& S, bool& ok) {
+                                      double kz, double umx, double umy, double umz, Step& S,
+                                      bool& ok) {
   auto div = [&](double a, double b) { return TRY ? xa_div_try(a, b, ok) : xa_div(a, b); };
   auto root = [&](double a) { return TRY ? xa_sqrt_try(a, ok) : xa_sqrt(a); };
   double t;
-  if (SMALL) t = xa_div_1p_try(F.hb, xa_gamma_ulps(xm), ok);
-  else t = div(F.hb, root(1.0 + xm));
+  if (SMALL) t = xa_div_1p_try(F.hb, xa_gamma_ulps3(umx, umy, umz, ok), ok);
+  else t = div(F.hb, root(1.0 + (umx * umx + umy * umy + umz * umz) * INV_C2));
   const double sf = div(xa_twice(t), 1.0 + t * t);
   const double upx = umx + umy * t, upy = umy - umx * t;
   S.unx = umx + upy * sf + kx;
   S.uny = umy - upx * sf + ky;
   S.unz = O.ez ? umz + kz : (dzero(umz) ? umz + F.h * 0.0 : umz);
-  S.u2n = S.unx * S.unx + S.uny * S.uny + S.unz * S.unz;
-  const double xn2 = S.u2n * INV_C2;
+  // (without energy bins nothing asks for u^2, and SMALL does not need it)
+  S.u2n = !SMALL || F.binned ? S.unx * S.unx + S.uny * S.uny + S.unz * S.unz : 0.0;
   double sc;
-  if (SMALL) {
-    ok = ok && bits(xn2) < X_SMALL;
-    sc = xa_div_1p_try(F.dt, xa_gamma_ulps(xn2), ok);
-  } else {
-    sc = div(F.dt, root(1.0 + xn2));
-  }
+  if (SMALL) sc = xa_div_1p_try(F.dt, xa_gamma_ulps3(S.unx, S.uny, S.unz, ok), ok);
+  else sc = div(F.dt, root(1.0 + S.u2n * INV_C2));
   S.dx = S.unx * sc;
   S.dy = S.uny * sc;
   S.dz = S.unz * sc;
@@ -321,6 +325,8 @@ __device__ bool start_flight(const Params& P, const OrbitDev& O, OPart& Q, Fligh
     if (b > 0) F.u2lo = edge[b];
     if (b < ntb - 1) F.u2hi = edge[b + 1];
   }
+  F.small = slow(Q.ux, Q.uy, Q.uz);
+  F.binned = F.u2lo >= 0.0 || F.u2hi < INFINITY;
   F.step = 0;
   F.cj = -1; F.cr = -1; F.cn = 0;
   F.rate = 0.0;
@@ -480,16 +486,20 @@ __device__ bool load(const Params& P, const OrbitDev& O, long long i, OPart& Q) 
   return true;
 }
 
-// Bound by the FP64 pipe: GB300 issues a warp's FP64 instruction in 64 cycles
-// of its scheduler, so a step costs its count of FP64 instructions and little
-// else.  The push's roots and quotients are therefore taken by
-// exact_arith.cuh (none or two FP64 instructions instead of eight to ten, the
-// same bits), the halvings and doublings on the exponent, the segment and
-// radial bin by integer and FP32 compares away from their edges, the rate per
-// segment kept while the segment lasts; the particles of a small generation
-// are spread over the schedulers (karl_run_orbit).  32768 ions at 2.5 T over
-// 3e-5 s: 340 ms -> 109 ms; 300 decays at 0.25 T (a few serial electrons):
-// 684 ms -> 564 ms.
+// Bound by the FP64 pipe when every scheduler has two warps or more (GB300
+// issues a warp's FP64 instruction in 64 cycles of its scheduler whatever its
+// lanes), by the step's chain of dependent instructions when few particles
+// run.  So the push's roots and quotients are taken by exact_arith.cuh (none or
+// two FP64 instructions instead of eight to ten, the same bits), gamma of slow
+// particles by integers, halvings and doublings on the exponent, segment and
+// radial bin by integer and FP32 compares away from their edges; the rate is
+// kept while the segment lasts; the usual step is straight code with one test;
+// the particles of a small generation are spread over the schedulers
+// (karl_run_orbit).  FP64 instructions of an ion's step 118 -> 38.  32768 ions
+// at 2.5 T over 3e-5 s: 340 ms -> 109 (roots, quotients, spread) -> 94
+// (straight code) -> 86 (gamma by integers); one ion's step 4.8 -> 2.4 us, one
+// electron's 4.8 -> 3.1 us; 300 decays at 0.25 T (a few serial electrons,
+// another seed) 473 -> 283 ms.
 __global__ void __launch_bounds__(512, 1) orbit_kernel(const Params P, const OrbitDev O) {
   if ((int)(threadIdx.x & 31) >= O.lanes) return;
   const double L = P.L;
@@ -529,12 +539,14 @@ __global__ void __launch_bounds__(512, 1) orbit_kernel(const Params P, const Orb
     const double kz = O.ez ? F.h * O.ez[F.js] : 0.0;
     const double umx = Q.ux + kx, umy = Q.uy + ky;
     const double umz = O.ez ? Q.uz + kz : (dzero(Q.uz) ? Q.uz + F.h * 0.0 : Q.uz);
-    const double xm = (umx * umx + umy * umy + umz * umz) * INV_C2;
     Step S;
     bool ok = true;
-    if (bits(xm) < X_SMALL) boris<true, true>(O, F, kx, ky, kz, umx, umy, umz, xm, S, ok);
-    else boris<true, false>(O, F, kx, ky, kz, umx, umy, umz, xm, S, ok);
-    if (!ok) boris<false, false>(O, F, kx, ky, kz, umx, umy, umz, xm, S, ok);
+    if (F.small) boris<true, true>(O, F, kx, ky, kz, umx, umy, umz, S, ok);
+    else boris<true, false>(O, F, kx, ky, kz, umx, umy, umz, S, ok);
+    if (!ok) {
+      boris<false, false>(O, F, kx, ky, kz, umx, umy, umz, S, ok);
+      F.small = F.small && slow(S.unx, S.uny, S.unz);
+    }
     const double unx = S.unx, uny = S.uny, unz = S.unz, u2n = S.u2n;
     const double dx = S.dx, dy = S.dy, dz = S.dz, ds = S.ds;
     const double hx = xa_half(dx), hy = xa_half(dy), hz = xa_half(dz);

@@ -51,13 +51,27 @@ CHK int chk_one(uint64_t i) {
   double x = chk_from(((long long)(1023 - 26 - (int)(r3 % 60)) << 52) | (long long)(r1 >> 12));
   if (near == 1) x = (double)(2 * (int)(r2 % 100000) + 1) * 1.1102230246251565e-16;   // ties
   const double y = 1.0 + x;
-  const int j = xa_gamma_ulps(x);
-  bad += xa_bits(xa_ieee_sqrt(y)) - XA_ONE != j;
+  const int j = (int)((xa_bits(xa_ieee_sqrt(y)) - XA_ONE));
   bad += !chk_same(xa_div_1p(a, j), xa_ieee_div(a, xa_ieee_sqrt(y)));
-  const double top = chk_from(((1023LL - 25) << 52) - 1 - (long long)(r2 & 0xffffffffffULL));
-  bad += xa_bits(xa_ieee_sqrt(1.0 + top)) - XA_ONE != xa_gamma_ulps(top);
   const int jt = (int)(r3 >> 40) >> (r3 & 15);
   bad += !chk_same(xa_div_1p(a, jt), xa_ieee_div(a, chk_from(XA_ONE + jt)));
-  bad += xa_gamma_ulps(0.0) != 0;
+  {
+    // components of a proper velocity, of like and unlike sizes
+    double u[3];
+    const uint64_t r[3] = {r1, r2, r3};
+    for (int c = 0; c < 3; ++c) {
+      const int spread = (int)((r3 >> 50) & 7) * 5;
+      u[c] = chk_from(((long long)(1023 + 8 - (int)(r[c] % (uint64_t)(1 + spread)) + (int)(r3 % 8)) << 52) |
+                      (long long)(chk_mix(r[c]) >> 12));
+      if ((r3 >> 44) % 16 == (uint64_t)c) u[c] = 0.0;
+      if (r[c] & 1024) u[c] = -u[c];
+    }
+    volatile double sx = u[0] * u[0], sy = u[1] * u[1], sz = u[2] * u[2];
+    volatile double sxy = sx + sy, s3 = sxy + sz;
+    volatile double x3 = s3 * (1.0 / (299792458.0 * 299792458.0));
+    bool ok = true;
+    const int j3 = xa_gamma_ulps3(u[0], u[1], u[2], ok);
+    if (ok) bad += xa_bits(xa_ieee_sqrt(1.0 + x3)) - XA_ONE != j3;
+  }
   return bad;
 }
