@@ -786,8 +786,17 @@ karl_status copy_out(karl_ctx* ctx, void* dst, const void* src, size_t bytes, bo
   return KARL_OK;
 }
 
-// The host outputs of a whole run, to be touched while its first pass runs.
-void touch_outputs(karl_ctx* ctx, const karl_tallies* out, size_t n) {
+// The host outputs of a whole run, to be touched while its first pass runs; the
+// context forgets them when the call ends, however it ends.
+struct TouchOutputs {
+  karl_ctx* ctx;
+  TouchOutputs(karl_ctx* c, const karl_tallies* out, size_t n);
+  ~TouchOutputs() { ctx->touch.clear(); }
+  TouchOutputs(const TouchOutputs&) = delete;
+  TouchOutputs& operator=(const TouchOutputs&) = delete;
+};
+
+TouchOutputs::TouchOutputs(karl_ctx* c, const karl_tallies* out, size_t n) : ctx(c) {
   ctx->touch.clear();
   if (out->on_device) return;
   try {
@@ -1074,7 +1083,7 @@ karl_status karl_run(karl_ctx* ctx, const karl_primaries* pr, const karl_run_opt
   s = stage_primaries(ctx, pr, st, &pz, &pe, &pmu, &psp);
   if (s) return s;
   bool pp = out->per_primary != nullptr && pr->n > 0;
-  touch_outputs(ctx, out, (size_t)pr->n);
+  const TouchOutputs touched(ctx, out, (size_t)pr->n);
   s = run_one_pass(ctx, pr, o, 1, pz, pe, pmu, psp, pp, st);
   if (s) return s;
   size_t nt = n_time(ctx);
@@ -1231,7 +1240,7 @@ karl_status karl_run_cycles(karl_ctx* ctx, const karl_primaries* pr, const karl_
     CK(cudaMemsetAsync(x.cum->p, 0, x.n * 8, st));
   }
   if (pp) CK(ctx->c_pp.ensure(nn));
-  touch_outputs(ctx, out, (size_t)pr->n);
+  const TouchOutputs touched(ctx, out, (size_t)pr->n);
   double kms = 0.0;
   int64_t colls = 0, flights = 0, parts = 0;
   const int64_t n = pr->n;
