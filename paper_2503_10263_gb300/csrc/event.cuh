@@ -845,7 +845,7 @@ __device__ __noinline__ int select_per_channel(const Params& P, int s, long long
       if (target < cum) { chs = c; break; }
     }
   } else {
-    const double nj = P.nseg[jc];
+    const double nj = P.nseg[(size_t)jc * P.nstep];
     double rtot = 0.0;
     for (int c = 0; c < nsc; ++c) {
       const int kk = P.sc[s][c];

@@ -284,6 +284,7 @@ inline void fill_params(Params& P, const karl_geometry& g, const ModelInfo& m, i
                         unsigned long long seed, int nq, double colmax) {
   std::memset(&P, 0, sizeof P);
   P.fstep = 1;
+  P.nstep = 1;
   P.nz = g.n_zbins;
   P.L = g.length_m;
   P.dz = g.length_m / g.n_zbins;

@@ -66,6 +66,7 @@ struct Params {
   // reads of a segment; multi-request kernel only
   const double* rec;       // [nz+1][4]
   int fstep;               // stride of the field tables below (2: pairs of column and rate)
+  int nstep;               // stride of nseg (4: in the records)
   int nq;
   double nq_over_colmax;   // nq / colgas[nz] (0 if the column is empty)
   float nq_over_colmax_f;  // same in FP32 (search hints only)

@@ -207,7 +207,7 @@ cudaError_t zero_by_copy(const karl_server* srv, void* dst, size_t bytes, cudaSt
 size_t footprint(const Sizes& z) {
   size_t b = 0;
   b += 3 * up(z.n * 8) + up(z.n);                                   // primaries
-  b += up(z.nz * 8) + up((z.nz + 1) * 32) + up((z.nq + 1) * 4);     // tables
+  b += up((z.nz + 1) * 32) + up((z.nq + 1) * 4);                    // tables
   const size_t tallies = up(z.nspec * 8) + 2 * up(z.nt * 8) + 2 * up(z.cross_rg * 8) +
                          up(z.rec * 8) + up(LEDGER * 8) + up(MAXCH * 8);
   b += 2 * tallies;                                                 // both passes
@@ -271,7 +271,6 @@ karl_status admit(karl_server* srv, Request& r) {
   double* pe = (double*)take(z.n * 8);
   double* pmu = (double*)take(z.n * 8);
   uint8_t* psp = (uint8_t*)take(z.n);
-  double* nseg = (double*)take(z.nz * 8);
   double* rec = (double*)take((z.nz + 1) * 32);
   int* ginv = (int*)take((z.nq + 1) * 4);
   char* tally0 = p;
@@ -308,7 +307,6 @@ karl_status admit(karl_server* srv, Request& r) {
     SCK(cudaMemcpyAsync(pmu, r.mu.data(), z.n * 8, cudaMemcpyHostToDevice, cs));
     SCK(cudaMemcpyAsync(psp, r.sp.data(), z.n, cudaMemcpyHostToDevice, cs));
   }
-  SCK(cudaMemcpyAsync(nseg, r.nseg.data(), z.nz * 8, cudaMemcpyHostToDevice, cs));
   SCK(cudaMemcpyAsync(rec, r.tabs.rec.data(), (z.nz + 1) * 32, cudaMemcpyHostToDevice, cs));
   SCK(cudaMemcpyAsync(ginv, r.tabs.ginv.data(), (z.nq + 1) * 4, cudaMemcpyHostToDevice, cs));
   SCK(zero_by_copy(srv, tally0, tally_bytes, cs));
@@ -324,7 +322,8 @@ karl_status admit(karl_server* srv, Request& r) {
   for (int k = 0; k < 2; ++k) {
     Params& P = d.P[k];
     fill_params(P, r.g, srv->model, k + 1, r.seed, r.tabs.nq, r.tabs.colmax);
-    P.nseg = nseg;
+    P.nseg = rec + 2;
+    P.nstep = 4;
     P.rec = rec;
     P.fstep = 2;
     P.ginv = r.tabs.nq > 0 ? ginv : nullptr;
