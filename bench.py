@@ -51,11 +51,11 @@ BYTES_PER_EVENT_FP32 = 80
 #     which also counts the lanes a divergent warp leaves idle;
 #   DRAM_BYTES: dram__bytes_read.sum + dram__bytes_write.sum, scaled to a launch
 #     by its collisions.
-FP64_OPS_PER_COLLISION = {"fp64": 117.7, "fp32": 26.2}
-FP64_PIPE_CYCLES_PER_COLLISION = {"fp64": 77.0, "fp32": 27.7}
-DRAM_BYTES_PER_COLLISION = {"fp64": 0.157, "fp32": 0.242}
+FP64_OPS_PER_COLLISION = {"fp64": 119.2, "fp32": 27.3}
+FP64_PIPE_CYCLES_PER_COLLISION = {"fp64": 74.4, "fp32": 22.3}
+DRAM_BYTES_PER_COLLISION = {"fp64": 0.112, "fp32": 0.113}
 FP64_OPS_PER_SM_CYCLE = 2
-THREADS_PER_INSTRUCTION = {"fp64": 24.2, "fp32": 22.6}   # smsp__thread_inst_executed_per_inst_executed
+THREADS_PER_INSTRUCTION = {"fp64": 25.3, "fp32": 24.6}   # smsp__thread_inst_executed_per_inst_executed
 WORKLOAD = ("config2: 1e7 decays (1e7 beta e- + 1e7 thermal T2+), parabolic profile with "
             "5e21 m^-2 column, L = 10 m, 1000 z segments, 7 e- channels + T2+ clustering + "
             "e-/ion recombination, two passes")
@@ -612,9 +612,10 @@ WORKLOAD_ORBIT = ("orbit ions: full-orbit Boris mover at B = 2.5 T with a radial
                   "ion elastic scattering; lifetime cap 1e-4 s (about 3.5e4 steps per ion)")
 # Per Boris step of the orbit kernel (ncu, profiles/orbit_kernel_ions_counters.md):
 # FP64 add/mul/fma thread-instructions with the predicate on, and SM-cycles
-# the FP64 pipe was busy
-FP64_OPS_PER_STEP = 118.1
-FP64_PIPE_CYCLES_PER_STEP = 91.8
+# the FP64 pipe was busy (of a run a quarter of this size, whose warps lose
+# more lanes at the end: an upper bound here)
+FP64_OPS_PER_STEP = 38.4
+FP64_PIPE_CYCLES_PER_STEP = 53.9
 
 
 def orbit_measure(n_ions: int, steps: int, warmup: int, timeout: float, cpu_seconds: float,
