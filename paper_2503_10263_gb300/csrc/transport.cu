@@ -68,8 +68,9 @@ __device__ __forceinline__ void stage_tables(const Params& P, double* at) {
 // offsets of the block's shared memory, without a pointer; nothing takes the
 // particle's address but copies on the rare paths, which are out of line.
 // (With the parameters behind a shared-memory reference and the particle in
-// local memory, the FP32 form's pass 1 took 28.2 ms at 1e5 decays, 26.1 now;
-// 3e5 decays at 3.1e21 m^-2 47 and 42 ms.  The FP64 form, held by its FP64
+// local memory, the FP32 form's pass 1 took 28.2 ms at 1e5 decays, 26.1
+// without, and 25.7 since the conversions are done on the bits; 3e5 decays at
+// 3.1e21 m^-2 47, 42 and 40.5 ms.  The FP64 form, held by its FP64
 // instructions, gained 1 %.)
 template <bool F32, bool STAGED>
 __global__ void __launch_bounds__(512, 1)
