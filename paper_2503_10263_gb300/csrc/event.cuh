@@ -326,6 +326,23 @@ struct WarpQueue {
 // queue, so the products of the next events still find room).
 constexpr int RING_BATCH = WQ / 2;
 
+// The `more` particles of a claim that the warp's lanes have no room for, from
+// ring position pos on, go to its queue behind the qleft there; the queue's new
+// length.  A cell that does not come in time ends the run on its error, and
+// then none of them joins the queue: a place that was not read holds whatever
+// lay there, and an event on it would index the tables with that.
+__device__ __forceinline__ int ring_to_queue(const Ring& R, Control* ctl, unsigned long long pos,
+                                             int more, WarpQueue& Q, int qleft,
+                                             unsigned long long deadline) {
+  const int lane = threadIdx.x & 31;
+  const bool got = lane >= more || ring_get(R, ctl, pos + lane, Q.s[qleft + lane], deadline);
+  if (__all_sync(FULL, got)) qleft += more;
+  __syncwarp();
+  if (lane == 0) Q.top = qleft;
+  __syncwarp();
+  return qleft;
+}
+
 // Collisions in the rare channels (ionization with its products, clustering,
 // charge exchange) cost as much FP64 work as a whole ordinary event, and a warp pays that cost
 // in full for a single lane.  A lane that selects one parks its particle here

@@ -657,14 +657,8 @@ __global__ void __launch_bounds__(256, 2) multi_kernel(SlotDesc* D, SlotCtl* C, 
         }
       }
       credit += __popc(__ballot_sync(FULL, born_dead));
-      if (got > k) {                               // more than the idle lanes: to the queue
-        const int more = got - k;
-        if (lane < more) ring_get(R, ctl, base + k + lane, Q.s[qleft + lane], deadline);
-        qleft += more;
-        __syncwarp();
-        if (lane == 0) Q.top = qleft;
-        __syncwarp();
-      }
+      if (got > k)                                  // more than the idle lanes: to the queue
+        qleft = ring_to_queue(R, ctl, base + k, got - k, Q, qleft, deadline);
     }
 
     // ---- parked rare collisions: once enough have gathered, free lanes and

@@ -389,14 +389,8 @@ __global__ void __launch_bounds__(512, 1)
         }
       }
       credit += __popc(__ballot_sync(FULL, born_dead));
-      if (rgot > k) {                              // more than the idle lanes: to the queue
-        const int more = rgot - k;
-        if (lane < more) ring_get(R, ctl, rbase + k + lane, Q.s[qleft + lane], deadline);
-        qleft += more;
-        __syncwarp();
-        if (lane == 0) Q.top = qleft;
-        __syncwarp();
-      }
+      if (rgot > k)                                  // more than the idle lanes: to the queue
+        qleft = ring_to_queue(R, ctl, rbase + k, rgot - k, Q, qleft, deadline);
     }
 
     // ---- parked rare collisions: once enough have gathered, free lanes and
