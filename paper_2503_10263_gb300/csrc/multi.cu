@@ -175,8 +175,10 @@ __device__ __forceinline__ int task_units(const SlotDesc& d, int phase) {
 
 // The end of pass p of request s: publish the work that follows it.  One
 // lane; the request is alive until that work completes, so its generation is
-// current.
-__device__ void end_pass(SlotDesc* D, SlotCtl* C, MultiCtl* M, int s, int p) {
+// current.  Called where the lane sees the pass empty and not kept for the end
+// of its iteration: a lane can empty two passes in one, that of a primary born
+// dead and that of the parked particle it takes next.
+__device__ __noinline__ void end_pass(SlotDesc* D, SlotCtl* C, MultiCtl* M, int s, int p) {
   const int gen_bits = ld_acquire_i(&C[s].state) & ~0xff;
   const int from = gen_bits | (p == 1 ? SLOT_PASS1 : SLOT_PASS2);
   if (atomicCAS(&C[s].state, from, gen_bits | SLOT_TRANS) != from) return;
@@ -387,8 +389,6 @@ __global__ void __launch_bounds__(256, 2) multi_kernel(SlotDesc* D, SlotCtl* C, 
     if (o.excit) atomicAdd(led + L_LOSS_EXCIT, o.excit);
     o.flights = o.colls = o.recoil = o.excit = 0;
   };
-  // a pass this lane saw empty (by the death of a particle or a primary born dead)
-  int trigB = 0, tslotB = 0, tpassB = 1;
 
   for (long long iter = 0;; ++iter) {
     if ((iter & 15) == 0 || idle) {
@@ -648,7 +648,10 @@ __global__ void __launch_bounds__(256, 2) multi_kernel(SlotDesc* D, SlotCtl* C, 
               __threadfence();
               const unsigned long long o2 =
                   atomicAdd(&C[gslot].word[gpass - 1], (unsigned long long)0 - 1ULL);
-              if (pass_emptied(o2, 1ULL, D[gslot].n_prim)) { trigB = 1; tslotB = gslot; tpassB = gpass; }
+              if (pass_emptied(o2, 1ULL, D[gslot].n_prim)) {
+                __threadfence();
+                end_pass(D, C, M, gslot, gpass);
+              }
             } else {
               has = true;
             }
@@ -759,7 +762,10 @@ __global__ void __launch_bounds__(256, 2) multi_kernel(SlotDesc* D, SlotCtl* C, 
         __threadfence();                          // its tallies before its death
         const unsigned long long o2 =
             atomicAdd(&C[slot_of()].word[second()], (unsigned long long)0 - 1ULL);
-        if (pass_emptied(o2, 1ULL, D[slot_of()].n_prim)) { trigB = 1; tslotB = slot_of(); tpassB = second() ? 2 : 1; }
+        if (pass_emptied(o2, 1ULL, D[slot_of()].n_prim)) {
+          __threadfence();
+          end_pass(D, C, M, slot_of(), second() ? 2 : 1);
+        }
       }
       credit += __popc(__ballot_sync(FULL, died)) - (qtop - qleft);
       if (credit < 0) {
@@ -768,14 +774,6 @@ __global__ void __launch_bounds__(256, 2) multi_kernel(SlotDesc* D, SlotCtl* C, 
         credit = 0;
       }
     }
-
-    // ---- passes that just emptied: publish the work that follows ----
-    if (trigB) {
-      __threadfence();
-      end_pass(D, C, M, tslotB, tpassB);
-      trigB = 0;
-    }
-    __syncwarp();
 
     if (!busy) {
       // leave when the host has closed the session and every published
