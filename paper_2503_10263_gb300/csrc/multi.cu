@@ -757,6 +757,7 @@ __global__ void __launch_bounds__(256, 2) multi_kernel(SlotDesc* D, SlotCtl* C, 
           atomicAdd(Pl->chan_count + o.chan, (unsigned long long)__popc(grp));
       }
       o.chan = -1;
+      __syncwarp();                               // other lanes' counts before a lane's death
       if (died) {
         flush_sums();
         __threadfence();                          // its tallies before its death
