@@ -408,7 +408,7 @@ __global__ void __launch_bounds__(256, 2) multi_kernel(SlotDesc* D, SlotCtl* C, 
         // adopt requests the host has published since the last look
         unsigned long long pub = ld_acquire(&M->published);
         unsigned long long ad = ld_relaxed(&M->adopted);
-        while (ad < pub) {
+        while (ad < pub) {                       // (not once LEFT is set)
           const unsigned long long old = atomicCAS(&M->adopted, ad, ad + 1);
           if (old == ad) {
             const int s = (int)ld_acquire_i((const int*)&M->pubq[ad % MAX_SLOTS]);
@@ -778,13 +778,18 @@ __global__ void __launch_bounds__(256, 2) multi_kernel(SlotDesc* D, SlotCtl* C, 
 
     if (!busy) {
       // leave when the host has closed the session and every published
-      // request is done
+      // request is done (multi.cuh, LEFT)
       int done = 0;
       if (lane == 0) {
         if (credit > 0)
           atomicAdd((unsigned long long*)&ctl->active, (unsigned long long)(-(long long)credit));
-        done = ld_relaxed_i(&M->shutdown) &&
-               ld_relaxed(&M->done_count) >= ld_acquire(&M->published);
+        unsigned long long ad = ld_relaxed(&M->adopted);
+        if (!(ad & LEFT) && ld_relaxed_i(&M->shutdown) && ad == ld_acquire(&M->published) &&
+            ld_relaxed(&M->done_count) >= ad) {
+          const unsigned long long old = atomicCAS(&M->adopted, ad, ad | LEFT);
+          ad = old == ad ? ad | LEFT : old;
+        }
+        done = (ad & LEFT) != 0;
       }
       credit = 0;
       if (__shfl_sync(FULL, done, 0)) break;

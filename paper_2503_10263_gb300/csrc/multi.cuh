@@ -77,13 +77,21 @@ struct SlotDesc {
   int pad1;
 };
 
+// Leaving is one decision for the whole launch: the warp that finds the session
+// closed and every adopted request done sets this bit of the adopted count by a
+// compare-and-swap on the count it saw, and from then on no warp adopts and all
+// leave.  (Each warp for itself could leave a request published meanwhile to
+// warps that do not take primaries, or to a few.)  What was published and not
+// adopted is the next launch's, which starts with the bit cleared.
+constexpr unsigned long long LEFT = 1ULL << 63;
+
 struct MultiCtl {
   Control c;                             // shared ring, abort, error, counters; prim_next
                                          // here counts the unclaimed primaries and active the
                                          // particles held (both only steer the schedule)
   unsigned long long published;          // requests published by the host (sequence)
   char pad0[120];
-  unsigned long long adopted;            // requests adopted by the kernel
+  unsigned long long adopted;            // requests adopted by the kernel; LEFT once the launch leaves
   char pad1[120];
   unsigned long long done_count;
   char pad2[120];

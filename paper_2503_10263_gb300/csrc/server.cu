@@ -217,7 +217,10 @@ size_t footprint(const Sizes& z) {
   return b;
 }
 
-__global__ void k_ring_seq(unsigned long long* seq, unsigned long long cap) {
+// every cell free at its position; the last launch's leave (multi.cuh) undone
+__global__ void k_ring_seq(unsigned long long* seq, unsigned long long cap,
+                           unsigned long long* adopted) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) *adopted &= ~LEFT;
   for (unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; i < cap;
        i += (unsigned long long)gridDim.x * blockDim.x)
     seq[i] = i;
@@ -231,7 +234,7 @@ karl_status launch(karl_server* srv) {
                       srv->cstream));
   SCK(cudaMemsetAsync(srv->d_cancel, 0, sizeof(int), srv->cstream));
   // ring counters restart at 0, so every cell must be free at its position again
-  k_ring_seq<<<1024, 256, 0, srv->cstream>>>(srv->ring.seq, srv->ring.cap);
+  k_ring_seq<<<1024, 256, 0, srv->cstream>>>(srv->ring.seq, srv->ring.cap, &srv->d_M->adopted);
   SCK(cudaGetLastError());
   SCK(cudaStreamSynchronize(srv->cstream));
   const bool f32 = srv->opts.precision == KARL_FP32;
@@ -508,7 +511,7 @@ karl_status reap_launch(karl_server* srv) {
                      cudaMemcpyDeviceToHost) == cudaSuccess) {
         char b[256];
         snprintf(b, sizeof b, "; published %llu adopted %llu done %llu ring head %llu tail %llu",
-                 hm.published, hm.adopted, hm.done_count, hm.c.head, hm.c.tail);
+                 hm.published, hm.adopted & ~LEFT, hm.done_count, hm.c.head, hm.c.tail);
         detail += b;
         for (auto& kv : srv->reqs) {
           const Request& r = kv.second;
@@ -563,7 +566,7 @@ karl_status ensure_ring(karl_server* srv) {
   SCK(cudaMalloc(&R.seq, n * 8));
   R.cap = srv->ring_cap;
   R.mask = srv->ring_cap - 1;
-  k_ring_seq<<<1024, 256, 0, srv->cstream>>>(R.seq, R.cap);
+  k_ring_seq<<<1024, 256, 0, srv->cstream>>>(R.seq, R.cap, &srv->d_M->adopted);
   SCK(cudaGetLastError());
   SCK(cudaStreamSynchronize(srv->cstream));
   return KARL_OK;
