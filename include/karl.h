@@ -507,9 +507,9 @@ karl_status karl_server_create(const karl_xs* xs, const karl_server_opts* opts,
  * as karl_tally_layout gives for this geometry, owned by the caller and kept
  * valid until karl_server_poll reports the request done; per_primary is not
  * used.  n_passes as in karl_run_opts.  The request is admitted at once if a
- * slot and arena space are free, else when karl_server_poll or
- * karl_server_run_all has collected enough finished requests (a submit
- * collects none).
+ * slot and arena space are free, else as earlier requests finish: a poll, a
+ * run_all or a later submit collects those that have (a submit only while
+ * requests wait, and at most once in 25 ms).
  * Errors: KARL_EINVAL (bad geometry, primaries, buffers, more than 2^31 - 1
  * primaries, or a footprint larger than the whole budget), KARL_ENOMEM. */
 karl_status karl_server_submit(karl_server* srv, const karl_geometry* geom,

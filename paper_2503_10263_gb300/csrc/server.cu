@@ -9,6 +9,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <chrono>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -158,6 +159,7 @@ struct karl_server {
   cudaStream_t kstream = nullptr, cstream = nullptr;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;    // around the current launch
   bool running = false;
+  std::chrono::steady_clock::time_point looked;   // when the launch started or results were last copied
   unsigned long long seq = 0;                  // requests published so far
   std::vector<int> slot_req;                   // slot -> request index (-1 free)
   std::map<uint64_t, Request> reqs;
@@ -249,6 +251,7 @@ karl_status launch(karl_server* srv) {
                    srv->opts.block_size, bps, srv->kstream));
   SCK(cudaEventRecord(srv->ev1, srv->kstream));
   srv->running = true;
+  srv->looked = std::chrono::steady_clock::now();
   srv->stats.kernel_launches += 1;
   return KARL_OK;
 }
@@ -467,6 +470,7 @@ karl_status collect(karl_server* srv, Request& r) {
   srv->arena.release(r.off, r.bytes);
   srv->slot_req[r.slot] = -1;
   r.state = REQ_FINISHED;
+  srv->looked = std::chrono::steady_clock::now();
   srv->stats.completed += 1;
   return KARL_OK;
 }
@@ -572,8 +576,7 @@ karl_status ensure_ring(karl_server* srv) {
   return KARL_OK;
 }
 
-// collect finished requests (not while submitting: a submit copies no other
-// request's results back), then admit waiting ones in arrival order
+// collect finished requests, then admit waiting ones in arrival order
 karl_status progress(karl_server* srv, bool collecting = true) {
   karl_status st = reap_launch(srv);
   if (st && st != KARL_ECAPACITY) return st;
@@ -805,7 +808,14 @@ karl_status karl_server_submit(karl_server* srv, const karl_geometry* g, const k
   srv->reqs.emplace(r.id, std::move(r));
   srv->waiting.push_back(*req_id);
   srv->stats.submitted += 1;
-  return progress(srv, false);
+  // Where requests wait, finished ones make room for them, so that a client
+  // which only submits keeps the device busy.  Not in every submit: one takes
+  // 0.06 ms, copying a result back 0.2 ms or more, and a burst of submits is
+  // over sooner (96 in 6 ms) when the copies come after it.
+  const karl_status st = progress(srv, false);
+  constexpr auto gap = std::chrono::milliseconds(25);
+  if (st || srv->waiting.empty() || std::chrono::steady_clock::now() - srv->looked < gap) return st;
+  return progress(srv);
 }
 
 karl_status karl_server_poll(karl_server* srv, uint64_t req_id, int* done) {

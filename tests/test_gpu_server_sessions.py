@@ -46,3 +46,33 @@ def test_requests_published_while_the_launch_leaves(karl, slots, precision):
         assert st.completed == 6 * len(reqs) and st.kernel_launches >= 6
     finally:
         srv.close()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_a_client_that_only_submits_keeps_its_requests_moving(karl, precision):
+    # two slots, a request every 30 ms (several times what one takes), no poll
+    # until the end: finished requests make room for waiting ones
+    import time
+    reqs = [inputs.config2(1 + i % 3, seed=60 + i, column_m2=5e19, nz=20) for i in range(12)]
+    srv = karl.Server(reqs[0][0], precision=precision, max_slots=2, hbm_budget_bytes=1 << 28,
+                      timeout_s=20)
+    try:
+        ids = []
+        for i, (p, q) in enumerate(reqs):
+            ids.append(srv.submit(p, q, 9 + i))
+            time.sleep(0.03)
+        st = srv.stats()
+        srv.run_all()
+        got = [srv.poll(i) for i in ids]
+    finally:
+        srv.close()
+    assert st.admitted == len(reqs) and st.waiting == 0 and st.collected == 0
+    for i, (done, t) in enumerate(got):
+        ctx = karl.Context(reqs[i][0])
+        try:
+            ref = ctx.run(reqs[i][1], seed=9 + i, precision=precision, per_primary=False)
+        finally:
+            ctx.close()
+        assert done
+        for k in INTEGER:
+            np.testing.assert_array_equal(t[k], ref[k], err_msg=f"{k} of request {i}")
