@@ -52,7 +52,8 @@ XA_FN float xa_rsqrt(float x) {
 }
 XA_FN int xa_rint(float x) { return __float2int_rn(x); }
 XA_FN float xa_float(int n) { return __int2float_rn(n); }
-// out of line: taken by one operand in a thousand
+// out of line: taken by one operand in a thousand, and by those outside the
+// range treated
 static __device__ __noinline__ double xa_ieee_div(double a, double b) { return __ddiv_rn(a, b); }
 static __device__ __noinline__ double xa_ieee_sqrt(double a) { return __dsqrt_rn(a); }
 #else
@@ -103,7 +104,8 @@ constexpr float XA_TIE = 0.4995f;
 // error 2^-21.2) leaves q1 within 2^-42.9, below 2^10.1 units of the last
 // place, and the second correction's error is below 2^-11 units.  q0's
 // significand must keep eight FP32 units from its binade's ends, so the
-// corrections (four of them at most) stay within it.  Two FP64 instructions.
+// corrections (four of them at most) stay within it (a power of two over a
+// divisor next to one does not).  Two FP64 instructions.
 // xa_div_try clears ok instead of calling the IEEE division (its value is then
 // meaningless), for straight code with one test for many quotients and roots.
 XA_FN double xa_div_try(double a, double b, bool& ok) {
@@ -140,16 +142,20 @@ XA_FN double xa_div(double a, double b) {
 // the seed y ~ 1/sqrt(m) (rsqrt.approx, 2^-22.3 with the truncated operand)
 // and corrections residual x y/2 (the root's second-order term is in the
 // first one's relative error, 2^-20.9; the second one's is below 2^-11 units).
-// Two FP64 instructions.
+// Roots lie in [1, 2), so g0 is not let below 1.  Those of m = 1 + k 2^-52 with
+// k < 2^27 are 1 + floor(k/2) 2^-52 (see xa_gamma_ulps3; odd k lie next to a
+// midpoint and the corrections could not tell), the others are above 1 + 2^-26
+// and stay there through both corrections; below 2 the corrections keep eight
+// FP32 units.  Two FP64 instructions.
 XA_FN double xa_sqrt_try(double a, bool& ok) {
   const long long ba = xa_bits(a);
   const int e = (int)(ba >> 52);
   const int odd = (e & 1) ^ 1;                               // exponent e - 1023 odd
-  const double m = xa_dbl((ba & XA_MANT) | ((long long)(1023 + odd) << 52));
+  const long long bm = (ba & XA_MANT) | ((long long)(1023 + odd) << 52);
+  const double m = xa_dbl(bm);
   const float mf = xa_flt((xa_fbits(xa_top24(ba))) + (odd << 23));
   const float y = xa_rsqrt(mf);
-  const float g0f = xa_fmul(mf, y);                          // in [1, 2)
-  const int gm = xa_fbits(g0f) & 0x7fffff;
+  const float g0f = fmaxf(xa_fmul(mf, y), 1.0f);
   const float yu = xa_fmul(y, 2251799813685248.0f);          // y/2 x 2^52
   const double g0 = xa_from_f(g0f);
   const double r0 = xa_fma(-g0, g0, m);
@@ -160,9 +166,12 @@ XA_FN double xa_sqrt_try(double a, bool& ok) {
   const float c1 = xa_fmul(xa_trunc_f(r1), yu);
   const int n1 = xa_rint(c1);
   const float off = c1 - xa_float(n1);
-  ok = ok && (unsigned)(e - 523) < 1000u && g0f >= 1.0f &&
-       (unsigned)(gm - 8) < 0x7fffffu - 16u && off < XA_TIE && off > -XA_TIE;
-  return xa_dbl(b1 + n1 + ((long long)((e - odd - 1023) / 2) << 52));
+  const unsigned long long k = (unsigned long long)(bm - XA_ONE);
+  const bool near1 = k < (1ULL << 27);
+  ok = ok && (unsigned)(e - 523) < 1000u &&
+       (near1 || (xa_fbits(g0f) < 0x3ffffff8 && off < XA_TIE && off > -XA_TIE));
+  return xa_dbl((near1 ? XA_ONE + (long long)(k >> 1) : b1 + n1) +
+                ((long long)((e - odd - 1023) / 2) << 52));
 }
 XA_FN double xa_sqrt(double a) {
   bool ok = true;
@@ -177,11 +186,12 @@ XA_FN double xa_sqrt(double a) {
 // integer below.  So j = floor(k/2) = floor((x 2^52 + 1/2) / 2), ties included.
 // For x = RN(RN(RN(RN(ux^2) + RN(uy^2)) + RN(uz^2)) / c^2), gamma of a proper
 // velocity of components below 2^14 m/s, it comes from 30-bit fixed-point
-// components: their squares' sum S (an integer, rounded components: relative
-// error below 2^-26) times 2^52 / c^2 gives x 2^52 with the error of S; where
-// that reaches an integer that floor((x 2^52 + 1/2) / 2) turns on, or a
-// component is too large, ok is cleared.  (The FP64 chain's own roundings are
-// below 2^-50.)  No FP64 instruction, against six for the chain.
+// components: their squares' sum S (components rounded, so off by at most
+// fx + fy + fz + 1 <= sqrt(3 S) + 1, a relative error below 2^-28 as S >= 2^58)
+// times 2^52 / c^2 gives x 2^52 with the error of S; where twice that (2^-27)
+// reaches an integer that floor((x 2^52 + 1/2) / 2) turns on, or a component is
+// too large, ok is cleared.  (The FP64 chain's own roundings are below 2^-50.)
+// No FP64 instruction, against six for the chain.
 XA_FN unsigned long long xa_mulhi(unsigned long long a, unsigned long long b) {
 #ifdef __CUDACC__
   return __umul64hi(a, b);
@@ -203,17 +213,17 @@ XA_FN int xa_gamma_ulps3(double ux, double uy, double uz, bool& ok) {
   const unsigned long long hi = xa_mulhi(S, 0xCD3F69CF4136CC8FULL);
   const int s = 4 - 2 * (em - 1023 - 29);                    // x 2^52 = hi 2^-s
   const unsigned long long A = hi + (1ULL << ((s - 1) & 63)), mask = (2ULL << (s & 63)) - 1;
-  const unsigned long long rem = A & mask, err = (hi >> 24) + 16;
+  const unsigned long long rem = A & mask, err = (hi >> 27) + 16;
   ok = ok && em <= 1036 && s < 61 && rem > err && rem < mask - err;
   return (int)(A >> ((s + 1) & 63));
 }
 
-// a / (1 + j 2^-52), correctly rounded, for 0 <= j < 2^20 and a normal a: with
+// a / (1 + j 2^-52), correctly rounded, for 0 <= j < 2^21 and a normal a: with
 // the significand A = 2^52 a', the quotient is A - w, w = a' j (1 - j 2^-52 +
-// ...).  w is taken from the 31 upper fraction bits of a', off by at most
-// j 2^-31 for those and a' j^2 2^-52 <= j 2^-31 for the second order; if it is
-// nearer to a midpoint than twice that, or A - w is not in a's binade, ok is
-// cleared.  No FP64 instruction.
+// ...).  w is taken from the 31 upper fraction bits of a', too low by at most
+// j 2^-31 for the others and too high by a' j^2 2^-52 <= 2 j 2^-31 for the
+// second order; if it is nearer to a midpoint than 4 j 2^-31, or A - w is not
+// in a's binade, ok is cleared.  No FP64 instruction.
 XA_FN double xa_div_1p_try(double a, int j, bool& ok) {
   const long long ba = xa_bits(a);
   const unsigned a31 = ((unsigned)(ba >> 21) & 0x7fffffffu) | 0x80000000u;   // a' 2^31
@@ -221,7 +231,7 @@ XA_FN double xa_div_1p_try(double a, int j, bool& ok) {
   const long long n = (long long)(w >> 31);                  // w rounded
   const unsigned rest = (unsigned)w & 0x7fffffffu, near = 4u * (unsigned)j + 4u;
   const int e = (int)(ba >> 52) & 0x7ff;
-  ok = ok && (unsigned)j < (1u << 20) && (j == 0 || rest - near < 0x80000000u - 2 * near) &&
+  ok = ok && (unsigned)j < (1u << 21) && (j == 0 || rest - near < 0x80000000u - 2 * near) &&
        (ba & XA_MANT) >= n && e > 0 && e < 0x7ff;
   return xa_dbl(ba - n);
 }

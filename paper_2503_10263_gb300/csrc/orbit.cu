@@ -42,8 +42,11 @@ namespace {
 enum { EV_NONE = 0, EV_WALL = 1, EV_EXIT = 2, EV_CAP = 3, EV_COLL = 4, EV_EBIN = 5 };
 constexpr int DOM_REDRAW = 3;          // optical depths drawn anew after an energy-bin stop
 constexpr double INV_C2 = 1.0 / (C_LIGHT * C_LIGHT);
-constexpr long long U_SMALL = 0x40d0000000000000LL;   // 2^14 m/s
-constexpr long long ABS = 0x7fffffffffffffffLL;
+// Square of the proper speed below which gamma is taken from integers: these
+// hold to 9.1 km/s (j < 2^21).  Picoseconds a step of 32768 ions, by integers
+// and by the general form: 0.6 eV 274 and 357, 1 eV 292 and 370, 2 eV (8.0 km/s)
+// 325 and 392, 2.5 eV (8.9 km/s) 415 and 400.
+constexpr double U2_SMALL = 8500.0 * 8500.0;   // (m/s)^2
 
 // Comparisons of the step's tests on the bits of the doubles (integer
 // operations, the same outcomes as the floating-point compares for numbers:
@@ -231,7 +234,7 @@ struct Flight {
   double tau, acc, e0, s1, s3;
   double u2lo, u2hi;               // the flight's energy bin as bounds on u^2
   bool binned;                     // either is finite
-  bool small;                      // no component of u reaches 2^14 m/s (as last looked at)
+  bool small;                      // u^2 below U2_SMALL (as last looked at)
   unsigned long long step;
   int cj, cr;                      // cell of the current run of steps
   unsigned long long cn;
@@ -244,9 +247,8 @@ struct Flight {
   unsigned long long w1, w2, w3;   // uniforms of the collision
 };
 
-// No component reaches U_SMALL.
 __device__ __forceinline__ bool slow(double ux, double uy, double uz) {
-  return max(max(bits(ux) & ABS, bits(uy) & ABS), bits(uz) & ABS) < U_SMALL;
+  return ux * ux + uy * uy + uz * uz < U2_SMALL;
 }
 
 // The bounds of the particle's cell (they only change with it).
@@ -265,18 +267,21 @@ struct Step {
 
 // Boris push: half electric kick, magnetic rotation, half kick.  TRY: straight
 // code that clears ok where a quotient or root could not be settled.  SMALL:
-// components below 2^14 m/s (thermal ions), where gamma = 1 + j 2^-52 follows
-// from them by integers, and so do the quotients by it.
+// below U2_SMALL (thermal ions), where gamma = 1 + j 2^-52 follows from the
+// components by integers, and so do the quotients by it.  Without a magnetic
+// field the rotation's t and its quotient are the zero h B.
 template <bool TRY, bool SMALL>
 __device__ __forceinline__ void boris(const OrbitDev& O, const Flight& F, double kx, double ky,
                                       double kz, double umx, double umy, double umz, Step& S,
                                       bool& ok) {
   auto div = [&](double a, double b) { return TRY ? xa_div_try(a, b, ok) : xa_div(a, b); };
   auto root = [&](double a) { return TRY ? xa_sqrt_try(a, ok) : xa_sqrt(a); };
-  double t;
-  if (SMALL) t = xa_div_1p_try(F.hb, xa_gamma_ulps3(umx, umy, umz, ok), ok);
-  else t = div(F.hb, root(1.0 + (umx * umx + umy * umy + umz * umz) * INV_C2));
-  const double sf = div(xa_twice(t), 1.0 + t * t);
+  double t = F.hb, sf = F.hb;
+  if (!dzero(F.hb)) {
+    if (SMALL) t = xa_div_1p_try(F.hb, xa_gamma_ulps3(umx, umy, umz, ok), ok);
+    else t = div(F.hb, root(1.0 + (umx * umx + umy * umy + umz * umz) * INV_C2));
+    sf = div(xa_twice(t), 1.0 + t * t);
+  }
   const double upx = umx + umy * t, upy = umy - umx * t;
   S.unx = umx + upy * sf + kx;
   S.uny = umy - upx * sf + ky;
@@ -499,7 +504,11 @@ __device__ bool load(const Params& P, const OrbitDev& O, long long i, OPart& Q) 
 // at 2.5 T over 3e-5 s: 340 ms -> 109 (roots, quotients, spread) -> 94
 // (straight code) -> 86 (gamma by integers); one ion's step 4.8 -> 2.4 us, one
 // electron's 4.8 -> 3.1 us; 300 decays at 0.25 T (a few serial electrons,
-// another seed) 473 -> 283 ms.
+// another seed) 473 -> 283 ms.  Picoseconds a step of 32768 ions by energy,
+// with every step done twice where the straight code settled no root next to
+// one and no zero field, and now: thermal 218 -> 210, 1.5 eV 406 -> 310, 10 eV
+// 565 -> 446, 1 keV 495 -> 409, thermal without a field 620 -> 216; 4000
+// electrons of 0.1 eV 1601 -> 857, without a field 2040 -> 647.
 __global__ void __launch_bounds__(512, 1) orbit_kernel(const Params P, const OrbitDev O) {
   if ((int)(threadIdx.x & 31) >= O.lanes) return;
   const double L = P.L;
