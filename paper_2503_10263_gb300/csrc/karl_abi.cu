@@ -1785,16 +1785,20 @@ extern "C" karl_status karl_run_orbit(karl_ctx* ctx, const karl_orbit* ob,
     if ((s = upload(ctx, ctx->o_edge2, e2.data(), e2.size(), st))) return s;
     O.edge2 = ctx->o_edge2.p;
     // FP32 bounds 2^-19 inside the edges (the first bin reaches the axis, the
-    // last one is open), and of the wall
+    // last one is open), and of the wall.  Where a position can leave FP32's
+    // range, or a squared edge its normal numbers, they hold for no radius.
     const double in = 1.0 / 524288.0;
-    std::vector<float2> b2((size_t)ob->n_rbins);
-    for (int k = 0; k < ob->n_rbins; ++k) {
+    const double reach = ob->tube_radius_m +
+                         C_LIGHT * *std::max_element(ob->dt_s, ob->dt_s + NSP);
+    const bool f32_radii = reach < 0x1p120 && ob->tube_radius_m / ob->n_rbins > 0x1p-55;
+    std::vector<float2> b2((size_t)ob->n_rbins, make_float2(INFINITY, -INFINITY));
+    for (int k = 0; k < ob->n_rbins && f32_radii; ++k) {
       b2[k].x = k == 0 ? -1.0f : (float)(e2[k] * (1.0 + in));
       b2[k].y = k == ob->n_rbins - 1 ? INFINITY : (float)(e2[k + 1] * (1.0 - in));
     }
     if ((s = upload(ctx, ctx->o_bin2, b2.data(), b2.size(), st))) return s;
     O.bin2 = ctx->o_bin2.p;
-    O.R2_lo = (float)(O.R2 * (1.0 - in));
+    O.R2_lo = f32_radii ? (float)(O.R2 * (1.0 - in)) : -1.0f;
     // the smallest z of each segment floor(z inv_dz) within [0, L]
     std::vector<long long> ze(nz + 1);
     for (size_t j = 1; j < nz; ++j) {

@@ -55,3 +55,25 @@ def test_vacuum_steps_are_the_oracles(karl, species, b_t, e_r, e_z):
     for k in ("ledger", "per_primary", "time_z", "time_r", "cross_pos", "cross_neg", "rcross_out",
               "rcross_in", "wall", "spectrum", "end_state"):
         np.testing.assert_array_equal(g[k], o[k], err_msg=k)
+
+
+@pytest.mark.parametrize("radius,dt,x", [(0.05, 1e31, 0.01), (1e39, 3e30, 7e38), (3e-30, 1e-38, 1e-30),
+                                         (1e-17, 1e-26, 3e-18)])
+def test_lengths_beyond_fp32(karl, radius, dt, x):
+    # the step tells wall and radial bin by FP32 squares where these are far
+    # from an edge; lengths whose squares or values leave FP32 take the exact way
+    prob = _vacuum(length=1.0, nz=7)
+    orb = inputs.Orbit(b_t=0.0, dt_s=np.full(4, dt), tube_radius_m=radius, n_rbins=6, max_steps=40)
+    n = 16
+    a = np.linspace(0.0, 0.9, n)
+    pr = _prims(x * a, 0.5 * x * a, np.linspace(0.1, 0.9, n), _energy(5e8, inputs.T2P),
+                np.where(np.arange(n) % 2, 0.0, 1e-4), 0.0, inputs.T2P)
+    ctx = karl.Context(prob)
+    try:
+        g = ctx.run_orbit(orb, pr, seed=4)
+    finally:
+        ctx.close()
+    o = oracle.orbit_run(prob, orb, pr, seed=4, n_threads=4)
+    for k in ("ledger", "per_primary", "time_r", "cross_pos", "cross_neg", "rcross_out", "rcross_in",
+              "wall", "spectrum", "end_state"):
+        np.testing.assert_array_equal(g[k], o[k], err_msg=k)
