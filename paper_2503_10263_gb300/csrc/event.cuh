@@ -119,10 +119,7 @@ template <> struct RT<false> {
     return eq >= 0 && eq < (1LL << 53) ? u53_scaled((unsigned long long)eq, 24)
                                        : (double)eq * (1.0 / 16777216.0);
   }
-  // trunc(RN(de 2^24 + 1/2)) for de >= 0, from the bits: with t = trunc(de 2^25)
-  // it is (t + 1) / 2 rounded down, and 1 for the one value just below 2^-25
-  // whose sum with 1/2 rounds up to 1 (at all others the sum's rounding does
-  // not reach the next integer: below 2^52 every integer and half is a double)
+  // trunc(RN(de 2^24 + 1/2)) for de >= 0, the truncation on the bits
   static __device__ __forceinline__ long long quant_de(R de) {   // de >= 0
     return trunc_nonneg(de * 16777216.0 + 0.5);
   }
@@ -1382,18 +1379,16 @@ __device__ __forceinline__ void event(const Params& P, const Params& PS, const C
     // impact energy for a target at rest): lab polar angle and energy transfer
     const R g = par<F32>(P.gam[s], P.gam_f[s]);
     const R g2 = par<F32>(P.gam2[s], P.gam2_f[s]);   // 2 g
-    R cchi, omc;                               // cos chi and 1 - cos chi
+    R cchi;
     const int ang = P.ch[k].ang;
     if (ang >= 0 && e >= (R)P.ang_thr[ang]) {
       cchi = table_cchi<F32>(PS, ang, e, T::u(w[2]));
-      omc = (R)1 - cchi;
     } else {
       cchi = (R)2 * T::u(w[2]) - (R)1;
-      omc = (R)1 - cchi;
     }
     R a;
     if constexpr (F32) a = fma_rn(g2, cchi, fma_rn(g, g, (R)1));
-    else a = fma_rn(g2, cchi, fma_rn(g, g, 1.0));      // g^2 + 1 rounded once, on the host
+    else a = fma_rn(g2, cchi, fma_rn(g, g, 1.0));
     const R ra = T::rsq(a);
     const R ct = mul_rn(cchi + g, ra);
     // energy given to the target, E - E' = E 2g(1 - cos chi)/(1+g)^2

@@ -569,9 +569,10 @@ size_t n_recomb(const karl_ctx* c) { return (size_t)NSP * c->nz; }
 // the occupancy maximum): one block of 512 threads per SM.  With at most 128
 // registers a thread that keeps as many warps resident as two blocks of 256,
 // and the single block's share of shared memory also holds the pass-2 field
-// tables.  Measured on the config-2 step against 256 x 2, both passes: 1e6
-// decays FP64 970 against 973 ms, FP32 463 against 476 ms; 1e5 decays FP64 116
-// against 118 ms, FP32 60.4 against 62.6 ms.
+// tables.  Measured on the config-2 step against 256 x 2, both passes: FP32
+// 1e6 decays 463 against 476 ms, 1e5 decays 60.4 against 62.6 ms; FP64 970
+// against 973 ms and 116 against 118 ms, which is no more than runs of one
+// shape differ by.
 int default_block(bool) { return 512; }
 
 karl_status ensure_ring(karl_ctx* ctx, unsigned long long cap) {
