@@ -142,12 +142,14 @@ XA_FN double xa_div(double a, double b) {
 // the seed y ~ 1/sqrt(m) (rsqrt.approx, 2^-22.3 with the truncated operand)
 // and corrections residual x y/2 (the root's second-order term is in the
 // first one's relative error, 2^-20.9; the second one's is below 2^-11 units).
-// Roots lie in [1, 2), so g0 is not let below 1.  Those of m = 1 + k 2^-52 with
-// k < 2^27 are 1 + floor(k/2) 2^-52 (see xa_gamma_ulps3; odd k lie next to a
-// midpoint and the corrections could not tell), the others are above 1 + 2^-26
-// and stay there through both corrections; below 2 the corrections keep eight
-// FP32 units.  Two FP64 instructions.
-XA_FN double xa_sqrt_try(double a, bool& ok) {
+// g0 must keep eight FP32 units from 1 and 2, as in xa_div.  Two FP64
+// instructions.
+// ONE: roots next to one as well (gamma of a slow particle; the others have no
+// use for them, and moving-target collisions were 3 % slower with it).  Those of
+// m = 1 + k 2^-52 with k < 2^27 are 1 + floor(k/2) 2^-52 (see xa_gamma_ulps3; odd k
+// lie next to a midpoint and the corrections could not tell); all others are
+// above 1 + 2^-26, and g0, not let below 1, stays there through both corrections.
+template <bool ONE> XA_FN double xa_sqrt_form(double a, bool& ok) {
   const long long ba = xa_bits(a);
   const int e = (int)(ba >> 52);
   const int odd = (e & 1) ^ 1;                               // exponent e - 1023 odd
@@ -155,7 +157,8 @@ XA_FN double xa_sqrt_try(double a, bool& ok) {
   const double m = xa_dbl(bm);
   const float mf = xa_flt((xa_fbits(xa_top24(ba))) + (odd << 23));
   const float y = xa_rsqrt(mf);
-  const float g0f = fmaxf(xa_fmul(mf, y), 1.0f);
+  const float g = xa_fmul(mf, y), g0f = ONE ? fmaxf(g, 1.0f) : g;
+  const int gm = xa_fbits(g0f) - 0x3f800000;                 // its place in [1, 2)
   const float yu = xa_fmul(y, 2251799813685248.0f);          // y/2 x 2^52
   const double g0 = xa_from_f(g0f);
   const double r0 = xa_fma(-g0, g0, m);
@@ -166,13 +169,15 @@ XA_FN double xa_sqrt_try(double a, bool& ok) {
   const float c1 = xa_fmul(xa_trunc_f(r1), yu);
   const int n1 = xa_rint(c1);
   const float off = c1 - xa_float(n1);
-  const unsigned long long k = (unsigned long long)(bm - XA_ONE);
-  const bool near1 = k < (1ULL << 27);
+  const bool even = off < XA_TIE && off > -XA_TIE;
+  const long long k = bm - XA_ONE, exp = (long long)((e - odd - 1023) / 2) << 52;
+  const bool near1 = ONE && k < (1LL << 27);
   ok = ok && (unsigned)(e - 523) < 1000u &&
-       (near1 || (xa_fbits(g0f) < 0x3ffffff8 && off < XA_TIE && off > -XA_TIE));
-  return xa_dbl((near1 ? XA_ONE + (long long)(k >> 1) : b1 + n1) +
-                ((long long)((e - odd - 1023) / 2) << 52));
+       (near1 || ((ONE ? gm < 0x7fffff - 8 : (unsigned)(gm - 8) < 0x7fffffu - 16u) && even));
+  return xa_dbl((near1 ? XA_ONE + (k >> 1) : b1 + n1) + exp);
 }
+XA_FN double xa_sqrt_try(double a, bool& ok) { return xa_sqrt_form<false>(a, ok); }
+XA_FN double xa_sqrt_one_try(double a, bool& ok) { return xa_sqrt_form<true>(a, ok); }
 XA_FN double xa_sqrt(double a) {
   bool ok = true;
   const double g = xa_sqrt_try(a, ok);

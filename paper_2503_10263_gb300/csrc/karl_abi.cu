@@ -1752,13 +1752,14 @@ extern "C" karl_status karl_run_orbit(karl_ctx* ctx, const karl_orbit* ob,
   OrbitDev O;
   std::memset(&O, 0, sizeof O);
   O.bz = ob->b_t;
+  O.no_b = ob->b_t == 0.0;
   O.R2 = ob->tube_radius_m * ob->tube_radius_m;
   O.r_scale = (double)ob->n_rbins / ob->tube_radius_m;
   O.er = ob->e_r_vm2;
   for (int sp = 0; sp < NSP; ++sp) {
     O.dt[sp] = ob->dt_s[sp];
     O.h[sp] = 0.5 * (ORBIT_CHARGE[sp] * C_LIGHT * C_LIGHT / ctx->mass[sp]) * ob->dt_s[sp];
-    O.hb[sp] = O.h[sp] * O.bz;
+    O.hb[sp] = O.no_b ? 0.0123456789 : O.h[sp] * O.bz;
   }
   O.e_cut = ctx->e_cut;
   O.spec_bin = ctx->spec_bin;

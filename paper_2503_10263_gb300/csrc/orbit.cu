@@ -42,10 +42,11 @@ namespace {
 enum { EV_NONE = 0, EV_WALL = 1, EV_EXIT = 2, EV_CAP = 3, EV_COLL = 4, EV_EBIN = 5 };
 constexpr int DOM_REDRAW = 3;          // optical depths drawn anew after an energy-bin stop
 constexpr double INV_C2 = 1.0 / (C_LIGHT * C_LIGHT);
+constexpr long long SIGN = (long long)0x8000000000000000ULL;
 // Square of the proper speed below which gamma is taken from integers: these
 // hold to 9.1 km/s (j < 2^21).  Picoseconds a step of 32768 ions, by integers
-// and by the general form: 0.6 eV 274 and 357, 1 eV 292 and 370, 2 eV (8.0 km/s)
-// 325 and 392, 2.5 eV (8.9 km/s) 415 and 400.
+// and by the general form: 0.6 eV 280 and 357, 1 eV 303 and 370, 2 eV (8.0 km/s)
+// 335 and 392, 2.5 eV (8.9 km/s) 415 and 405.
 constexpr double U2_SMALL = 8500.0 * 8500.0;   // (m/s)^2
 
 // Comparisons of the step's tests on the bits of the doubles (integer
@@ -269,19 +270,24 @@ struct Step {
 // code that clears ok where a quotient or root could not be settled.  SMALL:
 // below U2_SMALL (thermal ions), where gamma = 1 + j 2^-52 follows from the
 // components by integers, and so do the quotients by it.  Without a magnetic
-// field the rotation's t and its quotient are the zero h B.
+// field the rotation's t and its quotient are the zero h B (selected: a branch
+// around the quotients took 1 % of an electron's step).
 template <bool TRY, bool SMALL>
 __device__ __forceinline__ void boris(const OrbitDev& O, const Flight& F, double kx, double ky,
                                       double kz, double umx, double umy, double umz, Step& S,
                                       bool& ok) {
   auto div = [&](double a, double b) { return TRY ? xa_div_try(a, b, ok) : xa_div(a, b); };
   auto root = [&](double a) { return TRY ? xa_sqrt_try(a, ok) : xa_sqrt(a); };
-  double t = F.hb, sf = F.hb;
-  if (!dzero(F.hb)) {
-    if (SMALL) t = xa_div_1p_try(F.hb, xa_gamma_ulps3(umx, umy, umz, ok), ok);
-    else t = div(F.hb, root(1.0 + (umx * umx + umy * umy + umz * umz) * INV_C2));
-    sf = div(xa_twice(t), 1.0 + t * t);
-  }
+  auto gamma = [&](double u2) {
+    const double g2 = 1.0 + u2 * INV_C2;
+    return TRY ? xa_sqrt_one_try(g2, ok) : xa_sqrt(g2);
+  };
+  double t;
+  if (SMALL) t = xa_div_1p_try(F.hb, xa_gamma_ulps3(umx, umy, umz, ok), ok);
+  else t = div(F.hb, gamma(umx * umx + umy * umy + umz * umz));
+  double sf = div(xa_twice(t), 1.0 + t * t);
+  const double zero = xa_dbl((bits(F.h) ^ bits(O.bz)) & SIGN);
+  if (O.no_b) t = sf = zero;
   const double upx = umx + umy * t, upy = umy - umx * t;
   S.unx = umx + upy * sf + kx;
   S.uny = umy - upx * sf + ky;
@@ -290,7 +296,7 @@ __device__ __forceinline__ void boris(const OrbitDev& O, const Flight& F, double
   S.u2n = !SMALL || F.binned ? S.unx * S.unx + S.uny * S.uny + S.unz * S.unz : 0.0;
   double sc;
   if (SMALL) sc = xa_div_1p_try(F.dt, xa_gamma_ulps3(S.unx, S.uny, S.unz, ok), ok);
-  else sc = div(F.dt, root(1.0 + S.u2n * INV_C2));
+  else sc = div(F.dt, gamma(S.u2n));
   S.dx = S.unx * sc;
   S.dy = S.uny * sc;
   S.dz = S.unz * sc;
@@ -506,9 +512,9 @@ __device__ bool load(const Params& P, const OrbitDev& O, long long i, OPart& Q) 
 // electron's 4.8 -> 3.1 us; 300 decays at 0.25 T (a few serial electrons,
 // another seed) 473 -> 283 ms.  Picoseconds a step of 32768 ions by energy,
 // with every step done twice where the straight code settled no root next to
-// one and no zero field, and now: thermal 218 -> 210, 1.5 eV 406 -> 310, 10 eV
-// 565 -> 446, 1 keV 495 -> 409, thermal without a field 620 -> 216; 4000
-// electrons of 0.1 eV 1601 -> 857, without a field 2040 -> 647.
+// one and no zero field, and now: thermal 218 -> 210, 1.5 eV 406 -> 322, 10 eV
+// 565 -> 441, 1 keV 495 -> 419, thermal without a field 620 -> 244; 4000
+// electrons of 0.1 eV 1601 -> 858, without a field 2040 -> 864.
 __global__ void __launch_bounds__(512, 1) orbit_kernel(const Params P, const OrbitDev O) {
   if ((int)(threadIdx.x & 31) >= O.lanes) return;
   const double L = P.L;

@@ -49,7 +49,8 @@ struct OrbitDev {
   double er;                    // radial field per metre (V/m^2)
   double dt[NSP];               // Boris time step per species
   double h[NSP];                // q dt / 2m per species (m/s per V/m)
-  double hb[NSP];               // h B
+  double hb[NSP];               // h B, an ordinary number without a magnetic field
+  int no_b;                     // B is zero
   double e_cut, spec_bin;       // energies in eV
   double inv_dz;                // n_zbins / L (segment of z: floor(z inv_dz))
   double e_max;                 // top of the energy grid (eV)

@@ -50,7 +50,7 @@ extern "C" int rates(double u, long long n, double num0, long long* settled) {
     const Vec v = direction((uint64_t)i, u * (1 + 1e-3 * unit(chk_mix(3 * i))));
     const double y = one_plus(v), g = std::sqrt(y), num = num0 * (1 + unit(chk_mix(5 * i)));
     bool r = true, d = true, gi = true, di = true;
-    const double gt = xa_sqrt_try(y, r);
+    const double gt = xa_sqrt_one_try(y, r);
     const double qt = xa_div_try(num, g, d);
     const int j = xa_gamma_ulps3(v.x, v.y, v.z, gi);
     const long long jg = xa_bits(g) - XA_ONE;
@@ -58,7 +58,7 @@ extern "C" int rates(double u, long long n, double num0, long long* settled) {
     bad += (r && gt != g) + (d && qt != num / g) + (gi && j != jg) + (di && qi != num / g);
     settled[0] += r; settled[1] += d; settled[2] += gi; settled[3] += di;
     bool p = true;
-    const double t = xa_div_try(num, xa_sqrt_try(y, p), p), t2 = t * t;
+    const double t = xa_div_try(num, xa_sqrt_one_try(y, p), p), t2 = t * t;
     const double sf = xa_div_try(xa_twice(t), 1.0 + t2, p);
     if (p) bad += sf != 2.0 * t / (1.0 + t2);
     settled[4] += p;
@@ -73,7 +73,7 @@ extern "C" int roots_near_one(long long n) {
       const double a = xa_dbl(XA_ONE + k * 37 + (((long long)2 * e) << 52));
       const double b = xa_dbl(XA_ONE + (2LL << 52) - 1 - k + (((long long)2 * e) << 52));
       bool ok = true;
-      const double g = xa_sqrt_try(a, ok);
+      const double g = xa_sqrt_one_try(a, ok);
       // past 2^27 a root may lie in the tie band
       bad += ok ? g != std::sqrt(a) : k * 37 < (1LL << 27);
       bad += xa_sqrt(b) != std::sqrt(b);
