@@ -611,11 +611,8 @@ WORKLOAD_ORBIT = ("orbit ions: full-orbit Boris mover at B = 2.5 T with a radial
                   "segments; thermal T2+ born over the cross section, T2+ -> T3+ clustering, "
                   "ion elastic scattering; lifetime cap 1e-4 s (about 3.5e4 steps per ion)")
 # Per Boris step of the orbit kernel (ncu, profiles/orbit_kernel_ions_counters.md):
-# FP64 add/mul/fma thread-instructions with the predicate on, and SM-cycles
-# the FP64 pipe was busy (of a run a quarter of this size, whose warps lose
-# more lanes at the end: an upper bound here)
-FP64_OPS_PER_STEP = 38.4
-FP64_PIPE_CYCLES_PER_STEP = 53.9
+# FP64 add/mul/fma thread-instructions with the predicate on
+FP64_OPS_PER_STEP = 38.3
 
 
 def orbit_measure(n_ions: int, steps: int, warmup: int, timeout: float, cpu_seconds: float,
@@ -656,9 +653,7 @@ def orbit_measure(n_ions: int, steps: int, warmup: int, timeout: float, cpu_seco
                        "peak": peak / 1e9, "unit": "G FP64 thread-ops/s",
                        "frac": FP64_OPS_PER_STEP * out["value"] / peak,
                        "ops_per_step": FP64_OPS_PER_STEP, "kernel": "karl::orbit_kernel",
-                       "traffic": None,
-                       "fp64_pipe_busy_frac": FP64_PIPE_CYCLES_PER_STEP * out["value"] /
-                       (152 * 2.07e9)}
+                       "traffic": None}
     if cpu_seconds > 0:
         import oracle
         threads = os.cpu_count() or 1
